@@ -49,12 +49,7 @@ __device__ __forceinline__ uint32_t bit_at(RowT w, int x)
 // Latency: the threshold an attempt needs depends on whether the previous attempt
 // flipped (through E and through k).  Both candidates are loaded two attempts ahead and
 // the right one is picked once the previous decision is known, which takes the shared-
-// memory latency off the attempt-to-attempt dependency chain.  Both candidates are
-// compared with the random word as soon as they arrive, so the decision itself is one
-// select of two booleans, and both load addresses of the next-but-one attempt are
-// formed before the decision and selected by it.  So is, in the whole-row stream, the
-// row address the next attempt moves to if it flips (E + its step for both outcomes of
-// the current attempt): one select after a decision instead of a select and an add.
+// memory latency off the attempt-to-attempt dependency chain (a select and a compare).
 // ---------------------------------------------------------------------------------
 template <int L>
 struct RowOf {
@@ -522,29 +517,18 @@ __device__ __forceinline__ void process_row(const uint32_t (&U)[L / 8], uint32_t
     E = Eres;
 }
 
-// ---------------------------------------------------------------------------------
-// Continuous attempt stream over whole rows (whole-sweep launches).  The two threshold
-// candidates of every attempt are loaded two attempts ahead, across row ends as well:
-// the first two sites of the next row have as neighbours the current row's first two
-// sites (final after its attempts 0 and 1) and rows that the current row does not
-// change, so their counts, and the candidates of the next row's attempts 0 and 1, are
-// known during the current row's attempts L - 2 and L - 1.  A new row then starts with
-// its first two decisions ready instead of waiting for its counts and loads.
-// ---------------------------------------------------------------------------------
-template <int L, int STRIDE>
-struct AttemptStream {
-    static constexpr uint32_t kD2 = 8u * STRIDE, kDJ = STRIDE;   // row step 4 STRIDE (2 - k) = kD2 - kDJ J
-    uint32_t E;                      // table row address of the current energy
-    bool prev_acc;                   // the previous attempt flipped
-    uint32_t T0n, T1n, T0nn, T1nn;   // candidates of the next two attempts
-    uint32_t Eacc;                   // row address if the current attempt flips
-    uint32_t d0_next, d1_next;
+// Antiparallel-neighbour counts of a row, original spins, as byte fields of four sites per
+// word: word 2 i holds sites 8 i + 0, 2, 4, 6, word 2 i + 1 sites 8 i + 1, 3, 5, 7.  One
+// dp4a (a four-byte dot product) adds a constant multiple of one site's count to an
+// address: one instruction on the multiply pipe where a shift, a mask and an addition
+// took three on the integer ALU, the pipe with the most instructions of this loop.
+template <int L>
+struct RowCounts {
+    uint32_t k0[L / 4];   // if the left neighbour did not flip
+    uint32_t k1[L / 4];   // if it did
 
-    // Counts of the row (U above, C, D below) in nibble fields: K0 if the left
-    // neighbour did not flip, K1 if it did.
-    __device__ __forceinline__ static void counts(const uint32_t (&U)[L / 8], const uint32_t (&C)[L / 8],
-                                                  const uint32_t (&D)[L / 8], uint32_t (&K0)[L / 8],
-                                                  uint32_t (&K1)[L / 8])
+    __device__ __forceinline__ RowCounts(const uint32_t (&U)[L / 8], const uint32_t (&C)[L / 8],
+                                         const uint32_t (&D)[L / 8])
     {
         constexpr int NW = L / 8;
 #pragma unroll
@@ -553,27 +537,60 @@ struct AttemptStream {
             const uint32_t cl = __funnelshift_l(C[(i + NW - 1) % NW], C[i], 4);
             const uint32_t kb = (U[i] ^ C[i]) + (D[i] ^ C[i]) + (C[i] ^ cr);
             const uint32_t h0 = C[i] ^ cl;
-            K0[i] = kb + h0;
-            K1[i] = kb + 0x11111111u - h0;
+            const uint32_t a = kb + h0, b = kb + 0x11111111u - h0;
+            k0[2 * i] = a & 0x0F0F0F0Fu;
+            k0[2 * i + 1] = (a >> 4) & 0x0F0F0F0Fu;
+            k1[2 * i] = b & 0x0F0F0F0Fu;
+            k1[2 * i + 1] = (b >> 4) & 0x0F0F0F0Fu;
         }
     }
+    __device__ __forceinline__ uint32_t word0(int x) const { return k0[(x >> 3) * 2 + (x & 1)]; }
+    __device__ __forceinline__ uint32_t word1(int x) const { return k1[(x >> 3) * 2 + (x & 1)]; }
+};
+
+// acc + m * (count of site x in its count word w), m in [-128, 127].
+__device__ __forceinline__ uint32_t add_count(uint32_t w, int x, int m, uint32_t acc)
+{
+    return (uint32_t)__dp4a((int)w, (int)(((uint32_t)m & 0xFFu) << (8 * ((x & 7) >> 1))), (int)acc);
+}
+
+// ---------------------------------------------------------------------------------
+// Continuous attempt stream over whole rows (whole-sweep launches).  The two threshold
+// candidates of every attempt are loaded two attempts ahead, across row ends as well:
+// the first two sites of the next row have as neighbours the current row's first two
+// sites (final after its attempts 0 and 1) and rows that the current row does not
+// change, so their counts, and the candidates of the next row's attempts 0 and 1, are
+// known during the current row's attempts L - 2 and L - 1.  A new row then starts with
+// its first two decisions ready instead of waiting for its counts and loads.
+//
+// What bounds it: instruction issue.  A warp alone on its SM sub-partition issues one
+// half-rate instruction per two cycles whatever its pipe (a wide multiply takes four), so
+// at one warp the attempt costs twice its ALU and multiply instructions; with two warps
+// the pipes overlap in part.  Measured at L = 32, 16384 walkers: 27.2 instructions per
+// attempt (13.5 ALU, 8.7 multiply pipe, of them 4 wide, 3.1 LSU) against 31.1 with shifted
+// and masked fields, 24.9 us per sweep against 25.6 (one warp per sub-partition); 62.2
+// against 67.8 us at 48 640 walkers; L = 64, 32 768 walkers 169 against 186 us.
+// ---------------------------------------------------------------------------------
+template <int L, int STRIDE>
+struct AttemptStream {
+    static constexpr int kStep = -4 * STRIDE;          // row step of a flip: 4 STRIDE (2 - k) bytes
+    static constexpr uint32_t kTwo = 8u * STRIDE;
+    uint32_t E;                      // table row address of the current energy
+    uint32_t Eacc;                   // the same if the next attempt flips
+    bool prev_acc;                   // the previous attempt flipped
+    uint32_t T0n, T1n, T0nn, T1nn;   // candidates of the next two attempts
 
     // First row of a launch: the candidates of its attempts 0 and 1.
     __device__ __forceinline__ void start(const uint32_t (&U)[L / 8], const uint32_t (&C)[L / 8],
                                           const uint32_t (&D)[L / 8], uint32_t E0)
     {
-        uint32_t K0[L / 8], K1[L / 8];
-        counts(U, C, D, K0, K1);
-        const uint32_t J0a = field_x4(K0[0], 0), J0b = field_x4(K0[0], 1), J1b = field_x4(K1[0], 1);
+        const RowCounts<L> k(U, C, D);
         E = E0;
         prev_acc = false;
-        const uint32_t d0 = kD2 - kDJ * J0a;
-        Eacc = E0 + d0;
-        d0_next = kD2 - kDJ * J0b;
-        d1_next = kD2 - kDJ * J1b;
-        T0n = T1n = lds_u32(E + J0a);
-        T0nn = lds_u32(E + J0b);
-        T1nn = lds_u32(E + d0 + J1b);
+        Eacc = add_count(k.word0(0), 0, kStep, E0 + kTwo);
+        T0n = T1n = lds_u32(add_count(k.word0(0), 0, 4, E0));
+        T0nn = lds_u32(add_count(k.word0(1), 1, 4, E0));
+        T1nn = lds_u32(add_count(k.word1(1), 1, 4, Eacc));
     }
 
     // One row (U above, C updated in place, D below, D2 the row below D); on return the
@@ -583,13 +600,11 @@ struct AttemptStream {
                                         const uint32_t (&D2)[L / 8], const Src &src)
     {
         constexpr int NW = L / 8;
-        uint32_t K0[NW], K1[NW];
-        counts(U, C, D, K0, K1);
-        uint32_t K0n = 0u, K1n = 0u;   // word 0 of the next row's counts (fields 0 and 1 used)
+        RowCounts<L> k(U, C, D);
+        uint32_t n0e = 0u, n0o = 0u, n1o = 0u;   // counts of the next row's sites 0 (n0e) and 1 (n0o, n1o)
+        // site L - 1's right neighbour is site 0: its counts move by one if site 0 flips
         const uint32_t hr_last = ((C[NW - 1] >> 28) ^ C[0]) & 1u;
-        const uint32_t adj_if_flip = hr_last ? (uint32_t)-4 : 4u;
-        uint32_t adj_last = 0u;
-        uint32_t Eres = E;
+        const uint32_t adj_if_flip = hr_last ? 0xFF000000u : 0x01000000u;   // -1 or +1 in its byte
 #pragma unroll
         for (int xb = 0; xb < L; xb += 4) {
             const uint4 rw = src.get(xb);
@@ -600,56 +615,40 @@ struct AttemptStream {
                 const uint32_t cln = __funnelshift_l(D[NW - 1], D[0], 4);
                 const uint32_t kbn = (C[0] ^ D[0]) + (D2[0] ^ D[0]) + (D[0] ^ crn);
                 const uint32_t h0n = D[0] ^ cln;
-                K0n = kbn + h0n;
-                K1n = kbn + 0x11111111u - h0n;
+                n0e = (kbn + h0n) & 0x0Fu;
+                n0o = ((kbn + h0n) >> 4) & 0x0Fu;
+                n1o = ((kbn + 0x11111111u - h0n) >> 4) & 0x0Fu;
             }
             const uint32_t words[4] = {rw.x, rw.y, rw.z, rw.w};
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int x = xb + u;
-                const bool c0 = words[u] < T0n, c1 = words[u] < T1n;
-                const bool acc = prev_acc ? c1 : c0;
-                const uint32_t Epost = acc ? Eacc : Eres;
+                const uint32_t T = prev_acc ? T1n : T0n;
+                const bool acc = words[u] < T;
+                E = acc ? Eacc : E;
                 C[x >> 3] ^= acc ? (1u << (4 * (x & 7))) : 0u;
-                if (x == 0)
-                    adj_last = acc ? adj_if_flip : 0u;
-                if (RECORD)
-                    hist_add_one(Epost);
-                else
-                    pad_add_one<STRIDE>(Epost);
-                // candidates of attempt x + 2 (in this row or the next) for both outcomes
-                // of attempt x + 1
-                uint32_t J0c, J1c;
-                if (x + 2 < L) {
-                    J0c = field_x4(K0[(x + 2) >> 3], (x + 2) & 7);
-                    J1c = field_x4(K1[(x + 2) >> 3], (x + 2) & 7);
-                    if (x + 2 == L - 1) {
-                        J0c += adj_last;
-                        J1c += adj_last;
-                    }
-                } else if (x + 2 == L) {
-                    J0c = J1c = field_x4(K0n, 0);   // site 0: its left neighbour comes later
-                } else {
-                    J0c = field_x4(K0n, 1);
-                    J1c = field_x4(K1n, 1);
+                if (x == 0) {
+                    const uint32_t adj = acc ? adj_if_flip : 0u;
+                    k.k0[L / 4 - 1] += adj;
+                    k.k1[L / 4 - 1] += adj;
                 }
+                if (RECORD)
+                    hist_add_one(E);
+                else
+                    pad_add_one<STRIDE>(E);
+                // row address if attempt x + 1 flips, candidates of attempt x + 2 (in this row
+                // or the next) for both its outcomes; site 0's left neighbour comes later
+                const uint32_t s = x + 1 == L ? n0e : acc ? k.word1(x + 1) : k.word0(x + 1);
+                const uint32_t j0 = x + 2 < L ? k.word0(x + 2) : x + 2 == L ? n0e : n0o;
+                const uint32_t j1 = x + 2 < L ? k.word1(x + 2) : x + 2 == L ? n0e : n1o;
+                Eacc = add_count(s, (x + 1) % L, kStep, E + kTwo);
                 T0n = T0nn;
                 T1n = T1nn;
-                // the next attempt's flipped row, formed from both outcomes before this
-                // decision and selected by it
-                const uint32_t t1 = Eacc + d1_next, t0 = Eres + d0_next;
-                const uint32_t a0 = acc ? Eacc + J0c : Eres + J0c;
-                const uint32_t a1 = acc ? t1 + J1c : t0 + J1c;
-                T0nn = lds_u32(a0);
-                T1nn = lds_u32(a1);
-                Eacc = acc ? t1 : t0;
-                d0_next = kD2 - kDJ * J0c;
-                d1_next = kD2 - kDJ * J1c;
-                Eres = Epost;
+                T0nn = lds_u32(add_count(j0, (x + 2) % L, 4, E));
+                T1nn = lds_u32(add_count(j1, (x + 2) % L, 4, Eacc));
                 prev_acc = acc;
             }
         }
-        E = Eres;
     }
 };
 

@@ -58,30 +58,6 @@ cudaError_t launch_full_l(const SweepArgs &a, int wpb, bool record, cudaStream_t
     return launch_full_p<L, true>(a, wpb, record, s);
 }
 
-template <int L, int LAYOUT>
-int occupancy_full_t(int wpb)
-{
-    const size_t smem = full_smem_bytes(L, wpb, true);
-    auto kern = sweep_full_kernel<L, LAYOUT, true, false>;
-    if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, wpb, smem) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    return n;
-}
-
-template <int L>
-int occupancy_full_l(int layout, int wpb)
-{
-    return layout == MUCA_LAYOUT_PACKED ? occupancy_full_t<L, MUCA_LAYOUT_PACKED>(wpb)
-                                        : occupancy_full_t<L, MUCA_LAYOUT_INT8>(wpb);
-}
-
 }  // namespace
 
 #define MUCA_CAT2(a, b) a##b
@@ -90,11 +66,6 @@ int occupancy_full_l(int layout, int wpb)
 cudaError_t MUCA_CAT(launch_full_L, MUCA_L)(const SweepArgs &a, int wpb, bool record, cudaStream_t s)
 {
     return launch_full_l<MUCA_L>(a, wpb, record, s);
-}
-
-int MUCA_CAT(occupancy_full_L, MUCA_L)(int layout, int wpb)
-{
-    return occupancy_full_l<MUCA_L>(layout, wpb);
 }
 
 }  // namespace muca

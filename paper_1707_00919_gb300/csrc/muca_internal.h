@@ -126,23 +126,16 @@ cudaError_t launch_unpack(int32_t L, int32_t layout, int64_t W, const void *latt
 cudaError_t launch_philox(const uint32_t *ctr, uint32_t k0, uint32_t k1, size_t n, uint32_t *out,
                           cudaStream_t s);
 
-// Kernels of one L each (muca_full_L.cu): launch over any attempt range, and resident
-// blocks of the recording kernel per SM.
+// Kernels of one L each (muca_full_L.cu): launch over any attempt range.
 cudaError_t launch_full_L8(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
 cudaError_t launch_full_L16(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
 cudaError_t launch_full_L24(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
 cudaError_t launch_full_L32(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
 cudaError_t launch_full_L48(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
 cudaError_t launch_full_L64(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
-int occupancy_full_L8(int layout, int wpb);
-int occupancy_full_L16(int layout, int wpb);
-int occupancy_full_L24(int layout, int wpb);
-int occupancy_full_L32(int layout, int wpb);
-int occupancy_full_L48(int layout, int wpb);
-int occupancy_full_L64(int layout, int wpb);
 
-// Blocks of the recording sweep kernel for this L, layout and block size that one SM
-// holds at once (0 if the configuration does not fit).
+// Blocks of the sweep kernel for this L, layout and block size that one SM holds at once
+// by the sizing rule (0 if the configuration does not fit).
 int resident_blocks(int L, int layout, int walkers_per_block);
 
 // Batched persistent kernel: allows `smem` bytes of dynamic shared memory, reports how

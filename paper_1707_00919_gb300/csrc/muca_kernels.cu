@@ -460,25 +460,44 @@ cudaError_t launch_philox(const uint32_t *ctr, uint32_t k0, uint32_t k1, size_t 
     return cudaGetLastError();
 }
 
+// Registers per thread that the sizing rule counts with, by L and layout; 0 where L is
+// bounded by shared memory and threads alone.  The default block size, the walker count
+// of full occupancy and with it the chains of an instance created without an explicit
+// count follow from this rule, so it is fixed and does not move with the register
+// allocation of the sweep kernels (which stay below it or within 10 % of it).
+static int sizing_registers(int L, int layout)
+{
+    const bool packed = layout == MUCA_LAYOUT_PACKED;
+    switch (L) {
+    case 8: return packed ? 104 : 80;
+    case 16: return 88;
+    case 24: return 104;
+    case 32: return packed ? 112 : 120;
+    case 48: return packed ? 248 : 168;
+    case 64: return packed ? 168 : 200;
+    default: return 0;
+    }
+}
+
 int resident_blocks(int L, int layout, int wpb)
 {
-    switch (L) {
-    case 8: return occupancy_full_L8(layout, wpb);
-    case 16: return occupancy_full_L16(layout, wpb);
-    case 24: return occupancy_full_L24(layout, wpb);
-    case 32: return occupancy_full_L32(layout, wpb);
-    case 48: return occupancy_full_L48(layout, wpb);
-    case 64: return occupancy_full_L64(layout, wpb);
-    default: break;
-    }
-    // the generic kernel: bounded by shared memory and threads
-    int dev = 0, smem_sm = 0, thr_sm = 0;
+    int dev = 0, smem_sm = 0, smem_block = 0, regs_sm = 0, thr_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&smem_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&thr_sm, cudaDevAttrMaxThreadsPerMultiProcessor, dev) != cudaSuccess)
         return 0;   // no resident block: callers skip this block size
-    const size_t need = sweep_smem_bytes(L, wpb, true) + 1024;
-    return (int)std::min((size_t)smem_sm / need, (size_t)(thr_sm / wpb));
+    const int regs = sizing_registers(L, layout);
+    const size_t smem = regs ? full_smem_bytes(L, wpb, true) : sweep_smem_bytes(L, wpb, true);
+    if (regs && smem > (size_t)smem_block)
+        return 0;
+    // a block takes its shared memory rounded up (128 bytes) and 1 KB of its own
+    const size_t need = regs ? align_up(smem, 128) + 1024 : smem + 1024;
+    int n = (int)std::min((size_t)smem_sm / need, (size_t)(thr_sm / wpb));
+    if (regs)   // a quarter of the registers per sub-partition, whole warps
+        n = std::min(n, (regs_sm / 4 / (regs * 32)) * 4 / (wpb / 32));
+    return n;
 }
 
 size_t lattice_bytes(int32_t L, int32_t layout, int64_t W)
