@@ -146,7 +146,7 @@ int run_therm_record(muca_t h, uint64_t n_therm, uint64_t n_record, const uint32
     }
     muca::SweepArgs a = sweep_args(h, n_record, skip);
     a.n_therm = n_therm;
-    MUCA_CUDA(muca::launch_sweep_fused(a, h->wpb, h->stream), "sweep launch");
+    MUCA_CUDA(muca::launch_sweep(a, h->wpb, true, h->stream), "sweep launch");
     h->t += n_therm + n_record;
     return MUCA_OK;
 }
@@ -224,7 +224,7 @@ int default_walkers_per_block(int32_t L, int32_t layout, int64_t W)
     int best = 64;
     int64_t best_cost = INT64_MAX;
     for (int wpb = 32; wpb <= 256; wpb += 32) {
-        if (std::max(muca::sweep_smem_bytes(L, wpb, true), muca::full_smem_bytes(L, wpb, true)) > limit)
+        if (std::max(muca::sizing_smem_bytes(L, wpb), muca::full_smem_bytes(L, wpb, true)) > limit)
             continue;
         const int occ = muca::resident_blocks(L, layout, wpb);
         if (occ < 1)
@@ -268,7 +268,7 @@ int tune_options(const muca_options &in, muca_options *out)
             muca_options o = in;
             o.layout = lay;
             o.walkers_per_block = wpb != 0 ? wpb : default_walkers_per_block(in.L, lay, in.n_walkers);
-            if (std::max(muca::sweep_smem_bytes(o.L, o.walkers_per_block, true),
+            if (std::max(muca::sizing_smem_bytes(o.L, o.walkers_per_block),
                          muca::full_smem_bytes(o.L, o.walkers_per_block, true)) > muca::sweep_smem_limit())
                 continue;
             muca_t t = nullptr;
@@ -361,7 +361,7 @@ int muca_optimal_walkers(int32_t L, int32_t layout, int64_t *n_walkers, int32_t 
     int64_t best = 0;
     int32_t best_wpb = 0;
     for (int wpb = 32; wpb <= 256; wpb += 32) {
-        if (std::max(muca::sweep_smem_bytes(L, wpb, true), muca::full_smem_bytes(L, wpb, true)) > limit)
+        if (std::max(muca::sizing_smem_bytes(L, wpb), muca::full_smem_bytes(L, wpb, true)) > limit)
             continue;
         const int64_t per_sm = (int64_t)muca::resident_blocks(L, layout, wpb) * wpb;
         if (per_sm > best || (per_sm == best && per_sm > 0)) {
@@ -415,7 +415,7 @@ int muca_create_ex(const muca_options *opt, muca_t *out)
         wpb = default_walkers_per_block(L, opt->layout, opt->n_walkers);
     if (wpb < 32 || wpb > 256 || wpb % 32 != 0)
         return fail(MUCA_EINVAL, "walkers_per_block = %d: must be a multiple of 32 in [32, 256]", wpb);
-    const size_t smem = std::max(muca::sweep_smem_bytes(L, wpb, true), muca::full_smem_bytes(L, wpb, true));
+    const size_t smem = std::max(muca::sizing_smem_bytes(L, wpb), muca::full_smem_bytes(L, wpb, true));
     if (smem > muca::sweep_smem_limit())
         return fail(MUCA_EINVAL, "L = %d with %d walkers per block needs %zu bytes of shared memory", L, wpb,
                     smem);

@@ -24,7 +24,8 @@ struct muca_batch_s {
     size_t items_capacity = 0;
     int32_t n_items = 0;                  // items of the current member set
     std::vector<int32_t> members;         // instances in the current work list
-    size_t smem = 0;
+    size_t smem = 0;                      // of the largest member's table and rows
+    size_t smem_launch = 0;               // of a launch
     int grid = 0;
     cudaGraphExec_t exec = nullptr;       // one weight iteration of the current members
     uint64_t g_therm = 0, g_rec = 0;
@@ -132,7 +133,7 @@ int build_graph(muca_batch_t b)
             err = cudaMemsetAsync(h->d_hist, 0, sizeof(unsigned long long) * ((size_t)h->N + 1), b->stream);
     }
     if (err == cudaSuccess)
-        err = muca::launch_batch(b->d_args + nm, b->d_items, b->n_items, b->d_counter + 1, b->grid, b->smem, true,
+        err = muca::launch_batch(b->d_args + nm, b->d_items, b->n_items, b->d_counter + 1, b->grid, b->smem_launch, true,
                                  b->stream);
     for (int32_t j : b->members) {
         const muca_t h = b->inst[(size_t)j];
@@ -261,7 +262,7 @@ int batch_run_iteration(muca_batch_t b, const std::vector<int32_t> &active, cons
                                   b->stream),
                   "batch descriptor upload");
         MUCA_CUDA(cudaMemsetAsync(b->d_counter, 0, 2 * sizeof(uint32_t), b->stream), "work counter reset");
-        MUCA_CUDA(muca::launch_batch(b->d_args, b->d_items, b->n_items, b->d_counter, b->grid, b->smem, false,
+        MUCA_CUDA(muca::launch_batch(b->d_args, b->d_items, b->n_items, b->d_counter, b->grid, b->smem_launch, false,
                                      b->stream),
                   "batched thermalization");
         for (int32_t j : active) {
@@ -270,7 +271,7 @@ int batch_run_iteration(muca_batch_t b, const std::vector<int32_t> &active, cons
                       "histogram reset");
         }
         for (uint64_t done = 0;;) {
-            MUCA_CUDA(muca::launch_batch(b->d_args + nm, b->d_items, b->n_items, b->d_counter + 1, b->grid, b->smem,
+            MUCA_CUDA(muca::launch_batch(b->d_args + nm, b->d_items, b->n_items, b->d_counter + 1, b->grid, b->smem_launch,
                                          true, b->stream),
                       "batched recording");
             done += cap;
@@ -417,6 +418,7 @@ int muca_batch_create(const muca_t *instances, int32_t n, muca_batch_t *out)
             wpb -= 32;
         b->item_wpb.push_back(wpb);
         b->smem = std::max(b->smem, muca::full_smem_bytes(h->L, wpb, true, false, stride));
+        b->smem_launch = std::max(b->smem_launch, muca::launch_smem_bytes(h->L, wpb, false, stride));
         items += (size_t)((h->W + wpb - 1) / wpb);
     }
     b->items_capacity = items;
@@ -424,7 +426,7 @@ int muca_batch_create(const muca_t *instances, int32_t n, muca_batch_t *out)
     if (err == cudaSuccess)
         err = cudaEventCreateWithFlags(&b->staged, cudaEventDisableTiming);
     if (err == cudaSuccess)
-        err = muca::configure_batch(b->smem);
+        err = muca::configure_batch(b->smem_launch);
     if (err != cudaSuccess)
         return cleanup(cuda_fail(err, "batch set-up"));
     int dev = 0, sms = 0;
@@ -433,7 +435,7 @@ int muca_batch_create(const muca_t *instances, int32_t n, muca_batch_t *out)
         err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (err != cudaSuccess)
         return cleanup(cuda_fail(err, "multiprocessor count"));
-    const int occ = muca::batch_resident_blocks(b->smem);
+    const int occ = muca::batch_resident_blocks(b->smem_launch);
     if (occ < 1)
         return cleanup(fail(MUCA_EINVAL, "batched kernel does not fit an SM with %zu bytes of shared memory", b->smem));
     b->grid = sms * occ;
@@ -539,7 +541,7 @@ int muca_batch_sweep(muca_batch_t b, uint64_t n_sweeps, int record)
                   "batch descriptor upload");
         MUCA_CUDA(cudaEventRecord(b->staged, b->stream), "batch upload event");
         MUCA_CUDA(cudaMemsetAsync(b->d_counter, 0, sizeof(uint32_t), b->stream), "work counter reset");
-        MUCA_CUDA(muca::launch_batch(b->d_args, b->d_items, b->n_items, b->d_counter, b->grid, b->smem, record != 0,
+        MUCA_CUDA(muca::launch_batch(b->d_args, b->d_items, b->n_items, b->d_counter, b->grid, b->smem_launch, record != 0,
                                      b->stream),
                   "batched launch");
         n_sweeps -= chunk;
@@ -663,7 +665,7 @@ int muca_batch_sweep_noalloc(const muca_raw_instance *instances, int32_t n, uint
         while (wpb > 32 && muca::full_smem_bytes(r.L, wpb, true, true) > limit)
             wpb -= 32;
         wpbs[i] = wpb;
-        smem = std::max(smem, muca::full_smem_bytes(r.L, wpb, true, true));
+        smem = std::max(smem, muca::launch_smem_bytes(r.L, wpb, true));
         muca::SweepArgs &d = descs[i];
         d.L = r.L;
         d.layout = r.layout;

@@ -1,5 +1,5 @@
-// muca_full.cuh - the whole-sweep kernel for one lattice size; included by
-// muca_full_L.cu with MUCA_L defined, so that the six sizes compile in parallel.
+// muca_full.cuh - the sweep kernel for one lattice size; included by muca_full_L.cu with
+// MUCA_L defined, so that the sizes compile in parallel.
 #pragma once
 
 #include "muca_device.cuh"
@@ -11,51 +11,31 @@
 namespace muca {
 namespace {
 
-template <int L, int LAYOUT, bool RECORD, bool PARTIAL>
-__global__ void __launch_bounds__(256, 1) sweep_full_kernel(const SweepArgs a)
+template <int L, class Stream>
+__global__ void __launch_bounds__(256, 1) sweep_full_kernel(const SweepArgs a, const __grid_constant__ LaunchPlan plan,
+                                                            const bool record)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    // launch_sweep splits launches at the steps of counter word 1
-    sweep_block<L, RECORD, PARTIAL, false, kTableStride, true>(a, (int64_t)blockIdx.x * blockDim.x, blockDim.x, smem,
-                                                               LAYOUT);
+    sweep_block<L, false, kTableStride, Stream>(a, HostPlans{plan}, (int64_t)blockIdx.x * blockDim.x, blockDim.x, smem,
+                                                record);
 }
 
-template <int L, int LAYOUT, bool RECORD, bool PARTIAL>
-cudaError_t launch_full_t(const SweepArgs &a, int wpb, cudaStream_t s)
+template <int L, class Stream>
+cudaError_t launch_full_t(const SweepArgs &a, int wpb, bool record, cudaStream_t s)
 {
-    const size_t smem = full_smem_bytes(L, wpb, RECORD);
-    auto kern = sweep_full_kernel<L, LAYOUT, RECORD, PARTIAL>;
-    static size_t configured = 0;
-    if (smem > 48 * 1024 && smem > configured) {
-        cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = launch_smem_bytes(L, wpb);
+    auto kern = sweep_full_kernel<L, Stream>;
+    if (smem > 48 * 1024) {
+        const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (err != cudaSuccess)
             return err;
-        configured = smem;
     }
     const int64_t blocks = (a.W + wpb - 1) / wpb;
-    kern<<<(unsigned)blocks, wpb, smem, s>>>(a);
+    LaunchPlan plan;
+    plan.phase[0] = row_plan(L, a.t0, a.n_therm);
+    plan.phase[1] = row_plan(L, a.t0 + a.n_therm, a.n);
+    kern<<<(unsigned)blocks, wpb, smem, s>>>(a, plan, record);
     return cudaGetLastError();
-}
-
-template <int L, bool PARTIAL>
-cudaError_t launch_full_p(const SweepArgs &a, int wpb, bool record, cudaStream_t s)
-{
-    if (a.layout == MUCA_LAYOUT_PACKED)
-        return record ? launch_full_t<L, MUCA_LAYOUT_PACKED, true, PARTIAL>(a, wpb, s)
-                      : launch_full_t<L, MUCA_LAYOUT_PACKED, false, PARTIAL>(a, wpb, s);
-    return record ? launch_full_t<L, MUCA_LAYOUT_INT8, true, PARTIAL>(a, wpb, s)
-                  : launch_full_t<L, MUCA_LAYOUT_INT8, false, PARTIAL>(a, wpb, s);
-}
-
-// Any attempt range: whole sweeps from a sweep boundary take the kernel without the
-// partial-row path, everything else the one with it.
-template <int L>
-cudaError_t launch_full_l(const SweepArgs &a, int wpb, bool record, cudaStream_t s)
-{
-    const uint64_t N = (uint64_t)L * (uint64_t)L;
-    if (a.t0 % N == 0 && a.n % N == 0 && a.n_therm % N == 0)
-        return launch_full_p<L, false>(a, wpb, record, s);
-    return launch_full_p<L, true>(a, wpb, record, s);
 }
 
 }  // namespace
@@ -65,7 +45,7 @@ cudaError_t launch_full_l(const SweepArgs &a, int wpb, bool record, cudaStream_t
 
 cudaError_t MUCA_CAT(launch_full_L, MUCA_L)(const SweepArgs &a, int wpb, bool record, cudaStream_t s)
 {
-    return launch_full_l<MUCA_L>(a, wpb, record, s);
+    return launch_full_t<MUCA_L, AttemptStream<MUCA_L, kTableStride>>(a, wpb, record, s);
 }
 
 }  // namespace muca

@@ -18,8 +18,7 @@ constexpr int kHistSlot = 5;
 // within two rows of the current energy, so they stay inside the table even for
 // energies that do not match the lattices.
 constexpr int kTableGuard = 2;
-// Table row stride of the batched kernel: 6 words at L = 64 (the histogram word doubles
-// as the thermalization padding), so that 256 walkers fit next to the 4097-row table.
+// Table row stride of the batched kernel: 6 words at L = 64, so that 256 walkers fit next to the 4097-row table.
 __host__ __device__ constexpr int batch_table_stride(int L) { return L == 64 ? 6 : kTableStride; }
 
 // Device error word bits.
@@ -41,10 +40,54 @@ struct SweepArgs {
     const uint32_t *skip = nullptr;   // when set and nonzero at launch: the launch does nothing
     uint32_t walker0 = 0;             // global index of walker 0 (the Philox walker word is walker0 + w)
     // Thermalization attempts run before the launch's n recorded ones, from t0 (the
-    // recorded attempts then start at t0 + n_therm).  Only a recording whole-sweep launch
-    // (launch_sweep_fused) sets it; every other launch leaves it 0.
+    // recorded attempts then start at t0 + n_therm).  Only a recording launch in typewriter
+    // order sets it.
     uint64_t n_therm = 0;
 };
+
+// A range of attempts row by row: part of a first row, whole rows, part of a last row, all
+// with the same Philox counter word 1.
+struct RowPlan {
+    int32_t y0, x0, x0_end;        // first row, attempts [x0, x0_end) of it (none if equal)
+    int32_t y1;                    // first whole row
+    int32_t y2, tail;              // last row, attempts [0, tail) of it
+    uint32_t blk0, blk1, blk2;     // Philox blocks of column 0 of rows y0, y1 and y2
+    uint32_t c1;                   // counter word 1
+    uint64_t rows;                 // whole rows
+};
+
+struct LaunchPlan {
+    RowPlan phase[2];   // thermalization, the launch's own attempts
+};
+
+// The attempts from t0 on, at most n, that share t0's counter word 1 (t >> 34).
+__host__ __device__ inline uint64_t same_word1(uint64_t t0, uint64_t n)
+{
+    const uint64_t room = (((t0 >> 34) + 1) << 34) - t0;
+    return n < room ? n : room;
+}
+
+__host__ __device__ inline RowPlan row_plan(int L, uint64_t t0, uint64_t n)
+{
+    RowPlan p;
+    const int32_t i = (int32_t)(t0 % (uint64_t)(L * L));
+    p.y0 = p.y1 = i / L;
+    p.x0 = p.x0_end = i % L;
+    p.blk0 = p.blk1 = (uint32_t)((t0 - (uint64_t)p.x0) >> 2);
+    p.c1 = (uint32_t)(t0 >> 34);
+    if (p.x0 != 0) {
+        const uint64_t m = n < (uint64_t)(L - p.x0) ? n : (uint64_t)(L - p.x0);
+        p.x0_end = p.x0 + (int32_t)m;
+        n -= m;
+        p.y1 = p.y0 + 1 == L ? 0 : p.y0 + 1;
+        p.blk1 = p.blk0 + (uint32_t)(L / 4);
+    }
+    p.rows = n / (uint64_t)L;
+    p.tail = (int32_t)(n % (uint64_t)L);
+    p.y2 = (int32_t)(((uint64_t)p.y1 + p.rows) % (uint64_t)L);
+    p.blk2 = p.blk1 + (uint32_t)p.rows * (uint32_t)(L / 4);
+    return p;
+}
 
 // Device state of an iteration whose recursion runs on the device (muca_iterate_device).
 struct IterState {
@@ -82,33 +125,28 @@ struct BatchItem {
 
 constexpr int kBatchThreads = 256;   // threads per block of the batched kernel
 
-// Shared memory bytes a sweep launch with this many walkers per block needs.
-size_t sweep_smem_bytes(int L, int walkers_per_block, bool record);
+// Shared memory bytes that the sizing rule counts for an L without a register count of its
+// own (bit rows, thresholds and counts).
+size_t sizing_smem_bytes(int L, int walkers_per_block);
 
-// Shared memory bytes of the whole-sweep kernel (eight thresholds per energy).
+// Shared memory bytes of the sweep kernel's table and rows, by which block sizes are
+// chosen, and those of a launch (with the row of zeros).
 size_t full_smem_bytes(int L, int walkers_per_block, bool record, bool guard = false, int stride = kTableStride);
+size_t launch_smem_bytes(int L, int walkers_per_block, bool guard = false, int stride = kTableStride);
 
 // Largest dynamic shared memory a block may use on this device (bytes).
 size_t sweep_smem_limit();
 
-// Runs attempts [t0, t0 + n) of every walker in one launch: the kernel specialised for
-// L (L in {8, 16, 24, 32, 48, 64}; whole sweeps or, with its partial-row path, any
-// range), the generic kernel for other L.  Grid = ceil(W / walkers_per_block).
+// Runs a.n_therm thermalization attempts from a.t0 (recording launches only; may be 0),
+// then a.n attempts of every walker: one launch unless the range crosses a step of counter
+// word 1 (every 2^34 attempts).  Grid = ceil(W / walkers_per_block).
 cudaError_t launch_sweep(const SweepArgs &a, int walkers_per_block, bool record, cudaStream_t s);
-// a.n_therm thermalization attempts from a.t0, then a.n recorded ones: one launch of the
-// whole-sweep kernel where both are whole sweeps from a sweep boundary within one step of
-// counter word 1, else a thermalization launch and a recording launch.
-cudaError_t launch_sweep_fused(const SweepArgs &a, int walkers_per_block, cudaStream_t s);
 
 // Runs attempts [t0, t0 + n) of every walker in random shared site order (muca_random.cu;
 // any L, any attempt range; the given block size, or a smaller one that fits shared
 // memory).
 cudaError_t launch_random_sweep(const SweepArgs &a, int walkers_per_block, bool record, cudaStream_t s);
 size_t random_smem_bytes(int L, int walkers_per_block, bool record);
-
-// Routes whole sweeps to the generic kernel when false (used by tests that compare the
-// two kernels).
-void set_full_kernel_enabled(bool on);
 
 // Draws the initial spins (tag 1 stream) and their energy indices.
 cudaError_t launch_init(int32_t L, int32_t layout, int64_t W, uint64_t seed, uint32_t walker0, void *lattice,
@@ -127,11 +165,21 @@ cudaError_t launch_philox(const uint32_t *ctr, uint32_t k0, uint32_t k1, size_t 
                           cudaStream_t s);
 
 // Kernels of one L each (muca_full_L.cu): launch over any attempt range.
+cudaError_t launch_full_L4(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
 cudaError_t launch_full_L8(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
+cudaError_t launch_full_L12(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
 cudaError_t launch_full_L16(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
+cudaError_t launch_full_L20(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
 cudaError_t launch_full_L24(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
+cudaError_t launch_full_L28(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
 cudaError_t launch_full_L32(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
+cudaError_t launch_full_L36(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
+cudaError_t launch_full_L40(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
+cudaError_t launch_full_L44(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
 cudaError_t launch_full_L48(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
+cudaError_t launch_full_L52(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
+cudaError_t launch_full_L56(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
+cudaError_t launch_full_L60(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
 cudaError_t launch_full_L64(const SweepArgs &a, int wpb, bool record, cudaStream_t s);
 
 // Blocks of the sweep kernel for this L, layout and block size that one SM holds at once
@@ -140,18 +188,11 @@ int resident_blocks(int L, int layout, int walkers_per_block);
 
 // Batched persistent kernel: allows `smem` bytes of dynamic shared memory, reports how
 // many blocks of it an SM holds, and launches it over a work list (counter zeroed by
-// the caller before every launch; L must be one of 8, 16, 24, 32, 48, 64 and every
-// launch covers whole sweeps).
+// the caller before every launch; L must be one of 8, 16, 24, 32, 48, 64).
 cudaError_t configure_batch(size_t smem);
 int batch_resident_blocks(size_t smem);
 cudaError_t launch_batch(const SweepArgs *insts, const BatchItem *items, int32_t n_items, uint32_t *counter,
                          int grid, size_t smem, bool record, cudaStream_t s);
-// The recording instantiation of the batched kernel (its own translation unit).
-cudaError_t configure_batch_record(size_t smem);
-int batch_resident_blocks_record(size_t smem);
-cudaError_t launch_batch_record(const SweepArgs *insts, const BatchItem *items, int32_t n_items, uint32_t *counter,
-                                int grid, size_t smem, cudaStream_t s);
-
 // Allocation-free batched sweep (see muca_batch_sweep_noalloc in muca.h): descriptors,
 // walkers per item and the prefix sums of the work items per instance (prefix[0] = 0,
 // prefix[n] = all items, below 2^31) come from the host and travel in the launch

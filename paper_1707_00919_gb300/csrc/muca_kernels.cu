@@ -1,13 +1,7 @@
-// muca_kernels.cu - sm_103a kernels of the parallel multicanonical 2D Ising update
-// (Gross, Zierenberg, Weigel, Janke, arXiv:1707.00919, Sec. 2.3).
-//
-// One thread runs one walker (Sec. 2.3: one thread per walker, lattices interleaved so
-// that a warp's accesses to one site coalesce).  Inside a launch the walker's lattice
-// is bit-packed into shared memory, one word per row ([row][walker-in-block], so a
-// warp's row loads hit 32 consecutive words), the acceptance thresholds T[e][k] sit in
-// shared memory, random words come from an inline Philox4x32-10, and the visited
-// energies go run-length encoded into a per-block shared histogram that is added to the
-// global uint64 histogram once at the end of the launch.
+// muca_kernels.cu - the launch choice of the sweep kernels (muca_full.cuh) and the kernels
+// around them (initial spins, lattice packing and unpacking, the Philox test kernel) of the
+// parallel multicanonical 2D Ising update (Gross, Zierenberg, Weigel, Janke,
+// arXiv:1707.00919, Sec. 2.3).
 #include <algorithm>
 #include <cstdint>
 
@@ -15,146 +9,6 @@
 
 namespace muca {
 namespace {
-
-bool g_use_full_kernel = true;
-
-
-// ---------------------------------------------------------------------------------
-// Sweep kernel.  Template: row word type (uint32 for L <= 32, uint64 for L <= 64),
-// global lattice layout, and whether visited energies are recorded.
-// ---------------------------------------------------------------------------------
-template <typename RowT, int LAYOUT, bool RECORD>
-__global__ void __launch_bounds__(1024) sweep_kernel(const SweepArgs a)
-{
-    extern __shared__ __align__(16) unsigned char smem[];
-    if (a.skip && *a.skip)   // an iteration run on the device has finished
-        return;
-    const int L = a.L;
-    const int N = L * L;
-    const int nb = N + 1;
-    const int wpb = blockDim.x;
-    uint32_t *sT = reinterpret_cast<uint32_t *>(smem);
-    uint32_t *sH = sT + nb * 5;
-    RowT *sRows = reinterpret_cast<RowT *>(smem + align_up((size_t)(nb * 5 + (RECORD ? nb : 0)) * 4, 16));
-
-    const int tid = threadIdx.x;
-    const int64_t w = (int64_t)blockIdx.x * wpb + tid;
-    bool active = w < a.W;
-
-    for (int i = tid; i < nb * 5; i += wpb)
-        sT[i] = a.table[i];
-    if (RECORD)
-        for (int i = tid; i < nb; i += wpb)
-            sH[i] = 0u;
-
-    RowT *col = sRows + tid;   // this walker's rows: col[y * wpb]
-    int32_t e = 0;
-    if (active) {
-        if (LAYOUT == MUCA_LAYOUT_PACKED) {
-            const RowT *g = reinterpret_cast<const RowT *>(a.lattice);
-            for (int y = 0; y < L; ++y)
-                col[y * wpb] = g[(size_t)y * a.W + w];
-        } else {
-            const int8_t *g = reinterpret_cast<const int8_t *>(a.lattice);
-            for (int y = 0; y < L; ++y) {
-                RowT r = 0;
-#pragma unroll 16
-                for (int x = 0; x < L; ++x)   // unrolled: a row's loads are in flight together
-                    r |= (RowT)(g[(size_t)(y * L + x) * a.W + w] < 0) << x;
-                col[y * wpb] = r;
-            }
-        }
-        e = a.energy[w];
-        if (e < 0 || e > N) {
-            atomicOr(a.err, kErrEnergyRange);
-            active = false;
-        }
-    }
-    __syncthreads();
-
-    int32_t run_e = e;
-    uint32_t run_n = 0;
-    if (active) {
-        const uint32_t k0 = (uint32_t)a.seed, k1 = (uint32_t)(a.seed >> 32);
-        const uint32_t wid = a.walker0 + (uint32_t)w;
-        uint64_t t = a.t0;
-        const uint64_t tend = a.t0 + a.n;
-        while (t < tend) {
-            const int i = (int)(t % (uint64_t)N);
-            const int y = i / L;
-            const int x0 = i - y * L;
-            const uint64_t left = tend - t;
-            const int x1 = left < (uint64_t)(L - x0) ? x0 + (int)left : L;
-            const int yu = (y == 0) ? L - 1 : y - 1;
-            const int yd = (y == L - 1) ? 0 : y + 1;
-            const RowT U = col[yu * wpb];
-            RowT C = col[y * wpb];
-            const RowT D = col[yd * wpb];
-            // Vertical disagreements: bit x of VU/VD is fixed until site x itself is
-            // visited (a flip at x' != x leaves bit x alone), so one XOR per row serves
-            // every site of the row.
-            const RowT VU = U ^ C;
-            const RowT VD = D ^ C;
-            const uint64_t tb = t - (uint64_t)x0;   // attempt number of column 0
-            for (int xb = x0 & ~3; xb < x1; xb += 4) {
-                const uint64_t blk = (tb + (uint64_t)xb) >> 2;
-                const uint4 rw = philox4x32_10(make_uint4((uint32_t)blk, (uint32_t)(blk >> 32), wid, kTagMetropolis), k0, k1);
-                const uint32_t words[4] = {rw.x, rw.y, rw.z, rw.w};
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int x = xb + u;
-                    if (x < x0 || x >= x1)
-                        continue;
-                    const int xl = (x == 0) ? L - 1 : x - 1;
-                    const int xr = (x == L - 1) ? 0 : x + 1;
-                    const uint32_t sx = bit_at(C, x);
-                    const uint32_t k = bit_at(VU, x) + bit_at(VD, x) + (sx ^ bit_at(C, xl)) + (sx ^ bit_at(C, xr));
-                    const uint32_t thr = sT[e * 5 + (int)k];
-                    const bool acc = (words[u] < thr) | (thr == 0xFFFFFFFFu);
-                    if (acc) {
-                        C ^= (RowT)1 << x;
-                        e += 2 - (int)k;
-                    }
-                    if (RECORD) {
-                        if (e != run_e) {
-                            if (run_n)
-                                atomicAdd(&sH[run_e], run_n);
-                            run_e = e;
-                            run_n = 0u;
-                        }
-                        ++run_n;
-                    }
-                }
-            }
-            col[y * wpb] = C;
-            t += (uint64_t)(x1 - x0);
-        }
-        if (RECORD && run_n)
-            atomicAdd(&sH[run_e], run_n);
-    }
-    __syncthreads();
-    if (RECORD)
-        for (int i = tid; i < nb; i += wpb) {
-            const uint32_t v = sH[i];
-            if (v)
-                atomicAdd(&a.hist[i], (unsigned long long)v);
-        }
-    if (active) {
-        if (LAYOUT == MUCA_LAYOUT_PACKED) {
-            RowT *g = reinterpret_cast<RowT *>(a.lattice);
-            for (int y = 0; y < L; ++y)
-                g[(size_t)y * a.W + w] = col[y * wpb];
-        } else {
-            int8_t *g = reinterpret_cast<int8_t *>(a.lattice);
-            for (int y = 0; y < L; ++y) {
-                const RowT r = col[y * wpb];
-                for (int x = 0; x < L; ++x)
-                    g[(size_t)(y * L + x) * a.W + w] = bit_at(r, x) ? (int8_t)-1 : (int8_t)1;
-            }
-        }
-        a.energy[w] = e;
-    }
-}
 
 // ---------------------------------------------------------------------------------
 // Initial spins: +1 iff the top bit of the tag-1 word for attempt number t = site is
@@ -275,48 +129,28 @@ __global__ void philox_kernel(const uint32_t *ctr, uint32_t k0, uint32_t k1, siz
     out[4 * i + 3] = r.w;
 }
 
-// Dispatches a whole-sweep range to the kernel specialised for L; returns
-// cudaErrorNotSupported when L has no specialisation.
+// Dispatches a launch to the kernel for L.
 cudaError_t launch_full(const SweepArgs &a, int wpb, bool record, cudaStream_t s)
 {
     switch (a.L) {
+    case 4: return launch_full_L4(a, wpb, record, s);
     case 8: return launch_full_L8(a, wpb, record, s);
+    case 12: return launch_full_L12(a, wpb, record, s);
     case 16: return launch_full_L16(a, wpb, record, s);
+    case 20: return launch_full_L20(a, wpb, record, s);
     case 24: return launch_full_L24(a, wpb, record, s);
+    case 28: return launch_full_L28(a, wpb, record, s);
     case 32: return launch_full_L32(a, wpb, record, s);
+    case 36: return launch_full_L36(a, wpb, record, s);
+    case 40: return launch_full_L40(a, wpb, record, s);
+    case 44: return launch_full_L44(a, wpb, record, s);
     case 48: return launch_full_L48(a, wpb, record, s);
+    case 52: return launch_full_L52(a, wpb, record, s);
+    case 56: return launch_full_L56(a, wpb, record, s);
+    case 60: return launch_full_L60(a, wpb, record, s);
     case 64: return launch_full_L64(a, wpb, record, s);
     default: return cudaErrorNotSupported;
     }
-}
-
-bool has_full_kernel(int L) { return L == 8 || L == 16 || L == 24 || L == 32 || L == 48 || L == 64; }
-
-template <typename RowT, int LAYOUT, bool RECORD>
-cudaError_t launch_sweep_t(const SweepArgs &a, int wpb, cudaStream_t s)
-{
-    const size_t smem = sweep_smem_bytes(a.L, wpb, RECORD);
-    auto kern = sweep_kernel<RowT, LAYOUT, RECORD>;
-    static size_t configured = 0;   // dynamic smem limit already granted to this instantiation
-    if (smem > 48 * 1024 && smem > configured) {
-        cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (err != cudaSuccess)
-            return err;
-        configured = smem;
-    }
-    const int64_t blocks = (a.W + wpb - 1) / wpb;
-    kern<<<(unsigned)blocks, wpb, smem, s>>>(a);
-    return cudaGetLastError();
-}
-
-template <typename RowT>
-cudaError_t launch_sweep_row(const SweepArgs &a, int wpb, bool record, cudaStream_t s)
-{
-    if (a.layout == MUCA_LAYOUT_PACKED)
-        return record ? launch_sweep_t<RowT, MUCA_LAYOUT_PACKED, true>(a, wpb, s)
-                      : launch_sweep_t<RowT, MUCA_LAYOUT_PACKED, false>(a, wpb, s);
-    return record ? launch_sweep_t<RowT, MUCA_LAYOUT_INT8, true>(a, wpb, s)
-                  : launch_sweep_t<RowT, MUCA_LAYOUT_INT8, false>(a, wpb, s);
 }
 
 }  // namespace
@@ -325,15 +159,22 @@ size_t full_smem_bytes(int L, int wpb, bool record, bool guard, int stride)
 {
     (void)record;
     const size_t rows = (size_t)L * L + 1 + (guard ? 2 * kTableGuard : 0);
-    const size_t per_walker = L <= 32 ? (size_t)L * (L / 8) * 4 : (size_t)L * 8;
+    const size_t per_walker = L <= 32 ? (size_t)L * row_words(L) * 4 : (size_t)L * 8;
     return align_up(rows * (size_t)stride * 4, 16) + per_walker * (size_t)wpb;
 }
 
-size_t sweep_smem_bytes(int L, int wpb, bool record)
+size_t launch_smem_bytes(int L, int wpb, bool guard, int stride)
+{
+    const size_t rows = (size_t)L * L + 2 + (guard ? 2 * kTableGuard : 0);
+    const size_t per_walker = L <= 32 ? (size_t)L * row_words(L) * 4 : (size_t)L * 8;
+    return align_up(rows * (size_t)stride * 4, 16) + per_walker * (size_t)wpb;
+}
+
+size_t sizing_smem_bytes(int L, int wpb)
 {
     const size_t nb = (size_t)L * L + 1;
     const size_t row = L <= 32 ? 4 : 8;
-    return align_up((nb * 5 + (record ? nb : 0)) * 4, 16) + (size_t)L * wpb * row;
+    return align_up(nb * 6 * 4, 16) + (size_t)L * wpb * row;
 }
 
 size_t sweep_smem_limit()
@@ -345,54 +186,30 @@ size_t sweep_smem_limit()
     return (size_t)v;
 }
 
-static cudaError_t launch_generic(const SweepArgs &a, int wpb, bool record, cudaStream_t s)
-{
-    if (a.n == 0)
-        return cudaSuccess;
-    if (a.L <= 32)
-        return launch_sweep_row<uint32_t>(a, wpb, record, s);
-    return launch_sweep_row<unsigned long long>(a, wpb, record, s);
-}
-
 cudaError_t launch_sweep(const SweepArgs &a, int wpb, bool record, cudaStream_t s)
 {
-    if (a.n == 0 || a.W == 0)
+    if (a.W == 0 || (a.n == 0 && a.n_therm == 0))
         return cudaSuccess;
-    if (!has_full_kernel(a.L) || !g_use_full_kernel)
-        return launch_generic(a, wpb, record, s);
-    // the whole-sweep kernels keep Philox counter word 1 (t >> 34) fixed within a launch:
-    // a range that crosses a multiple of 2^34 runs as two launches
-    const uint64_t step = a.t0 >> 34;
-    if (((a.t0 + a.n - 1) >> 34) != step) {
-        SweepArgs first = a, second = a;
-        first.n = ((step + 1) << 34) - a.t0;
-        second.t0 = a.t0 + first.n;
-        second.n = a.n - first.n;
-        cudaError_t err = launch_full(first, wpb, record, s);
-        return err != cudaSuccess ? err : launch_sweep(second, wpb, record, s);
+    SweepArgs part = a;
+    if (a.n_therm > 0 && (a.t0 >> 34) != ((a.t0 + a.n_therm + a.n - 1) >> 34)) {
+        // not one launch: the thermalization by itself
+        part.n_therm = 0;
+        part.n = a.n_therm;
+        const cudaError_t err = launch_sweep(part, wpb, false, s);
+        if (err != cudaSuccess)
+            return err;
+        part.t0 = a.t0 + a.n_therm;
+        part.n = a.n;
+        return launch_sweep(part, wpb, record, s);
     }
-    return launch_full(a, wpb, record, s);
+    for (uint64_t left = a.n; left > 0; left -= part.n, part.t0 += part.n) {
+        part.n = a.n_therm > 0 ? left : same_word1(part.t0, left);
+        const cudaError_t err = launch_full(part, wpb, record, s);
+        if (err != cudaSuccess)
+            return err;
+    }
+    return cudaSuccess;
 }
-
-cudaError_t launch_sweep_fused(const SweepArgs &a, int wpb, cudaStream_t s)
-{
-    const uint64_t total = a.n_therm + a.n;
-    // one launch of the whole-sweep kernel (its whole-sweep form when both phases are
-    // whole sweeps from a sweep boundary, else its any-range form), counter word 1
-    // (t >> 34) the same for both phases
-    if (a.W > 0 && a.n_therm > 0 && a.n > 0 && has_full_kernel(a.L) && g_use_full_kernel && total > a.n &&
-        (a.t0 >> 34) == ((a.t0 + total - 1) >> 34))
-        return launch_full(a, wpb, true, s);
-    SweepArgs therm = a, rec = a;
-    therm.n = a.n_therm;
-    therm.n_therm = 0;
-    rec.t0 = a.t0 + a.n_therm;
-    rec.n_therm = 0;
-    const cudaError_t err = launch_sweep(therm, wpb, false, s);
-    return err != cudaSuccess ? err : launch_sweep(rec, wpb, true, s);
-}
-
-void set_full_kernel_enabled(bool on) { g_use_full_kernel = on; }
 
 cudaError_t launch_init(int32_t L, int32_t layout, int64_t W, uint64_t seed, uint32_t walker0, void *lattice,
                         int32_t *energy,
@@ -489,7 +306,7 @@ int resident_blocks(int L, int layout, int wpb)
         cudaDeviceGetAttribute(&thr_sm, cudaDevAttrMaxThreadsPerMultiProcessor, dev) != cudaSuccess)
         return 0;   // no resident block: callers skip this block size
     const int regs = sizing_registers(L, layout);
-    const size_t smem = regs ? full_smem_bytes(L, wpb, true) : sweep_smem_bytes(L, wpb, true);
+    const size_t smem = regs ? full_smem_bytes(L, wpb, true) : sizing_smem_bytes(L, wpb);
     if (regs && smem > (size_t)smem_block)
         return 0;
     // a block takes its shared memory rounded up (128 bytes) and 1 KB of its own

@@ -27,9 +27,8 @@ struct NoAllocLaunch {
 // kernel parameters may take 32 764 bytes (CUDA 12.1 and later)
 static_assert(sizeof(NoAllocLaunch) + sizeof(uint32_t *) <= 32764, "launch parameters too large");
 
-template <bool RECORD>
 __global__ void __launch_bounds__(256, 1) batch_noalloc_kernel(const __grid_constant__ NoAllocLaunch p,
-                                                               uint32_t *counter)
+                                                               uint32_t *counter, const bool record)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int32_t s_inst;
@@ -59,12 +58,12 @@ __global__ void __launch_bounds__(256, 1) batch_noalloc_kernel(const __grid_cons
         it.wpb = p.wpbs[i];
         it.wbase = wbase;
         switch (a.L) {
-        case 8: batch_item<8, RECORD, true>(a, it, smem); break;
-        case 16: batch_item<16, RECORD, true>(a, it, smem); break;
-        case 24: batch_item<24, RECORD, true>(a, it, smem); break;
-        case 32: batch_item<32, RECORD, true>(a, it, smem); break;
-        case 48: batch_item<48, RECORD, true>(a, it, smem); break;
-        case 64: batch_item<64, RECORD, true>(a, it, smem); break;
+        case 8: batch_item<8, true>(a, it, smem, record); break;
+        case 16: batch_item<16, true>(a, it, smem, record); break;
+        case 24: batch_item<24, true>(a, it, smem, record); break;
+        case 32: batch_item<32, true>(a, it, smem, record); break;
+        case 48: batch_item<48, true>(a, it, smem, record); break;
+        case 64: batch_item<64, true>(a, it, smem, record); break;
         default: break;
         }
     }
@@ -113,7 +112,7 @@ cudaError_t launch_batch_noalloc(const SweepArgs *descs, const int32_t *wpbs, co
     std::memcpy(p.wpbs, wpbs, sizeof(int32_t) * (size_t)n);
     std::memcpy(p.prefix, prefix, sizeof(int32_t) * (size_t)(n + 1));
     p.n = n;
-    auto kern = record ? batch_noalloc_kernel<true> : batch_noalloc_kernel<false>;
+    auto kern = batch_noalloc_kernel;
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess)
         return err;
@@ -131,7 +130,7 @@ cudaError_t launch_batch_noalloc(const SweepArgs *descs, const int32_t *wpbs, co
     err = cudaMemsetAsync(counter, 0, sizeof(uint32_t), s);
     if (err != cudaSuccess)
         return err;
-    kern<<<sms * occ, kBatchThreads, smem, s>>>(p, counter);
+    kern<<<sms * occ, kBatchThreads, smem, s>>>(p, counter, record);
     return cudaGetLastError();
 }
 

@@ -267,13 +267,8 @@ __global__ void __launch_bounds__(256) random_sweep_kernel(const SweepArgs a)
                 hist_count(E);
         };
         auto words = [&](uint64_t tt) {
-            // the walker's stream of typewriter order (tag 0) with the keys and the products
-            // that depend only on the walker and counter word 1 computed once (the launch
-            // keeps t >> 34 fixed)
-            const uint4 q = philox_walker_c1((uint32_t)(tt >> 2), pk);
-            // clamped so that "r < T" also accepts every attempt when T = 0xFFFFFFFF
-            return make_uint4(min(q.x, 0xFFFFFFFEu), min(q.y, 0xFFFFFFFEu), min(q.z, 0xFFFFFFFEu),
-                              min(q.w, 0xFFFFFFFEu));
+            // the walker's stream of typewriter order (the launch keeps t >> 34 fixed)
+            return block_words(block_head((uint32_t)(tt >> 2), pk), pk);
         };
         auto word_at = [](const uint4 &q, uint32_t u) { return u == 0 ? q.x : u == 1 ? q.y : u == 2 ? q.z : q.w; };
         int j = 0;

@@ -1,0 +1,93 @@
+"""Every lattice size and every form of the sweep kernel against the oracle, bit for bit:
+ranges cut at both ends, ranges inside one row, ragged warps, launches of many warps
+(direct threshold loads), batches whose range crosses a step of Philox counter word 1."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def M():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1707_00919_gb300 import muca
+    return muca
+
+
+def rand_weights(L, seed):
+    return np.cumsum(np.random.default_rng(seed).normal(0.0, 0.4, L * L + 1))
+
+
+@pytest.mark.parametrize("L", range(4, 65, 4))
+def test_every_size_and_cut(M, orc, L):
+    W, seed, N = 45, 7 + L, L * L
+    lnW = rand_weights(L, L)
+    # (thermalization, recorded) attempts: inside a row, cut at both ends, ending at a row's
+    # end, whole sweeps, a fused launch cut at both ends
+    plan = [(0, 3), (1, 0), (0, N + L + 2), (2 * L + 3, 0), (0, 2 * N), (N + 5, N + L - 1)]
+    s, e = orc.init(L, seed, W)
+    T = orc.build_table(L, lnW)
+    t = 0
+    with M.Muca(L, W, seed, layout=(L // 4) % 2) as m:
+        m.set_weights(lnW)
+        for therm, rec in plan:
+            m.thermalize_and_record(therm, rec)
+            orc.run(L, seed, s, e, T, t, therm, False)
+            Ho = orc.run(L, seed, s, e, T, t + therm, rec, True)
+            t += therm + rec
+            H = m.get_histogram()
+            assert np.array_equal(H, Ho if rec else np.zeros(N + 1, dtype=np.uint64))
+            assert np.array_equal(m.get_energies(), e)
+        assert m.attempt_counter == t
+        assert np.array_equal(m.get_lattice(), s)
+
+
+@pytest.mark.parametrize("L,extra", [(8, 0), (8, 45), (12, 45), (20, 31), (32, 45)])
+def test_many_warps(M, orc, L, extra):
+    """More than two warps per SM sub-partition: the form with direct loads."""
+    import torch
+    W = torch.cuda.get_device_properties(0).multi_processor_count * 8 * 32 + 32 + extra
+    seed, N = 3, L * L
+    lnW = rand_weights(L, 2 * L)
+    T = orc.build_table(L, lnW)
+    with M.Muca(L, W, seed, layout=1, walkers_per_block=32) as m:
+        m.set_weights(lnW)
+        m.thermalize_and_record(N + 5, 2 * L + 3)
+        H, e, lat = m.get_histogram(), m.get_energies(), m.get_lattice()
+    assert int(H.sum()) == W * (2 * L + 3)
+    # all walkers where the oracle is quick, else the first and the last ones
+    for w0, n in ([(0, W)] if L <= 12 else [(0, 64), (W - 77, 77)]):
+        s, eo = orc.init(L, seed, n, walker0=w0)
+        orc.run(L, seed, s, eo, T, 0, N + 5, False, walker0=w0)
+        Ho = orc.run(L, seed, s, eo, T, N + 5, 2 * L + 3, True, walker0=w0)
+        assert np.array_equal(lat[w0:w0 + n], s)
+        assert np.array_equal(e[w0:w0 + n], eo)
+        if n == W:
+            assert np.array_equal(H, Ho)
+
+
+def test_batch_across_counter_word(M):
+    """Ranges that cross t = 2^34 inside a batched launch equal the instances run alone."""
+    specs = [(8, 70), (24, 33), (64, 40)]
+    for back in (2, 100, 64 * 64 + 8):
+        alone, together = [], []
+        for out in (alone, together):
+            inst = [M.Muca(L, W, 5 + L) for L, W in specs]
+            for m, (L, _) in zip(inst, specs):
+                m.set_weights(rand_weights(L, L))
+                m.set_attempt_counter(2**34 - back)
+            if out is alone:
+                for m in inst:
+                    m.sweep(2, record=True)
+            else:
+                with M.Batch(inst) as b:
+                    b.sweep(2, record=True)
+            for m in inst:
+                out.append((m.get_histogram(), m.get_energies(), m.get_lattice(), m.attempt_counter))
+                m.close()
+        for x, y in zip(alone, together):
+            assert all(np.array_equal(p, q) for p, q in zip(x, y))
