@@ -524,6 +524,76 @@ struct AttemptStream {
     }
 };
 
+// ---------------------------------------------------------------------------------
+// The same rows without the look-ahead: each attempt loads its one threshold once the
+// attempt before it is decided.  The chain of an attempt (address, load, compare, select)
+// then holds the load's latency, which other warps have to cover, but an attempt is 22.5
+// instructions instead of 27.2.  The decision enters as a factor 0 or 1: the step of the
+// energy row and the flip bit are multiply-adds, on the pipe with room, where a select
+// each would load the ALU.  Measured at L = 32, 48 640 walkers (2.5 warps per SM
+// sub-partition) 55.7 us per sweep against 62.8 with the look-ahead; L = 16, 77 824 walkers
+// (4 warps) 18.1 against 20.9; at one warp 33 against 24.9, at two 41 and 41 (L = 32, 38 912
+// walkers): launches of more than two warps per sub-partition take it.
+// ---------------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t mad32(uint32_t a, uint32_t b, uint32_t c)
+{
+    uint32_t r;
+    asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+    return r;
+}
+
+template <int L, int STRIDE>
+struct DirectStream {
+    static constexpr int NW = row_words(L);
+    uint32_t E;   // table row address of the current energy
+
+    __device__ __forceinline__ void start(const uint32_t (&)[NW], const uint32_t (&)[NW], const uint32_t (&)[NW],
+                                          uint32_t E0)
+    {
+        E = E0;
+    }
+
+    // One row (U above, C updated in place, D below).
+    template <class Src>
+    __device__ __forceinline__ void row(const uint32_t (&U)[NW], uint32_t (&C)[NW], const uint32_t (&D)[NW],
+                                        const uint32_t (&)[NW], Src &src)
+    {
+        RowCounts<L> k(U, C, D);
+        const uint32_t adj_if_flip = RowCounts<L>::last_step(C);
+        uint32_t flips[NW];
+#pragma unroll
+        for (int i = 0; i < NW; ++i)
+            flips[i] = 0u;
+        uint32_t kw = k.word0(0);
+#pragma unroll
+        for (int xb = 0; xb < L; xb += 4) {
+            const uint4 rw = src.get(xb);
+            if (xb == L - 4)
+                src.advance();
+            const uint32_t words[4] = {rw.x, rw.y, rw.z, rw.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int x = xb + u;
+                const uint32_t T = lds_u32(add_count(kw, x, 4, E));
+                const uint32_t step = add_count(kw, x, -4 * STRIDE, 8u * STRIDE);
+                const bool acc = words[u] < T;
+                uint32_t m = acc ? 1u : 0u;
+                asm volatile("" : "+r"(m));   // kept as a number
+                E = mad32(m, step, E);
+                flips[x >> 3] = mad32(m, 1u << (4 * (x & 7)), flips[x >> 3]);
+                if (x == 0)
+                    k.add_to_last(acc ? adj_if_flip : 0u);
+                if (x + 1 < L)
+                    kw = acc ? k.word1(x + 1) : k.word0(x + 1);
+                hist_add_one(E);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < NW; ++i)
+            C[i] ^= flips[i];
+    }
+};
+
 // nrows whole rows of one walker as one continuous attempt stream, from row y (wrapping to
 // row 0 after row L - 1) whose column 0 lies in Philox block b.  Counter word 1 must stay
 // at pk.c1 for the whole range.  The row below the next one is loaded from shared memory

@@ -43,9 +43,10 @@ cudaError_t launch_full_t(const SweepArgs &a, int wpb, bool record, cudaStream_t
 #define MUCA_CAT2(a, b) a##b
 #define MUCA_CAT(a, b) MUCA_CAT2(a, b)
 
-cudaError_t MUCA_CAT(launch_full_L, MUCA_L)(const SweepArgs &a, int wpb, bool record, cudaStream_t s)
+cudaError_t MUCA_CAT(launch_full_L, MUCA_L)(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s)
 {
-    return launch_full_t<MUCA_L, AttemptStream<MUCA_L, kTableStride>>(a, wpb, record, s);
+    return ahead ? launch_full_t<MUCA_L, AttemptStream<MUCA_L, kTableStride>>(a, wpb, record, s)
+                 : launch_full_t<MUCA_L, DirectStream<MUCA_L, kTableStride>>(a, wpb, record, s);
 }
 
 }  // namespace muca
