@@ -16,7 +16,7 @@ LIB = os.path.join(PKG, "libmuca.so")
 SOURCES = (["muca_batch.cu", "muca_noalloc.cu"] + [f"muca_full_{L}.cu" for L in range(64, 0, -4)] +
            ["muca_random.cu", "muca_kernels.cu", "muca_iterate.cu", "muca_probe.cu", "muca_api.cu",
             "muca_api_iterate.cu", "muca_api_batch.cu"])
-HEADERS = ["muca_internal.h", "muca_device.cuh", "muca_full.cuh", "muca_math.cuh", "muca_host.h"]
+HEADERS = ["muca_internal.h", "muca_device.cuh", "muca_full.cuh", "muca_pair.cuh", "muca_math.cuh", "muca_host.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

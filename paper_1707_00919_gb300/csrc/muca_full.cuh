@@ -3,6 +3,7 @@
 #pragma once
 
 #include "muca_device.cuh"
+#include "muca_pair.cuh"
 
 #ifndef MUCA_L
 #error "define MUCA_L before including muca_full.cuh"
@@ -25,11 +26,10 @@ cudaError_t launch_full_t(const SweepArgs &a, int wpb, bool record, cudaStream_t
 {
     const size_t smem = launch_smem_bytes(L, wpb);
     auto kern = sweep_full_kernel<L, Stream>;
-    if (smem > 48 * 1024) {
-        const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (err != cudaSuccess)
-            return err;
-    }
+    static std::atomic<uint64_t> allowed{0};
+    const cudaError_t err = allow_smem(kern, allowed);
+    if (err != cudaSuccess)
+        return err;
     const int64_t blocks = (a.W + wpb - 1) / wpb;
     LaunchPlan plan;
     plan.phase[0] = row_plan(L, a.t0, a.n_therm);
@@ -43,10 +43,12 @@ cudaError_t launch_full_t(const SweepArgs &a, int wpb, bool record, cudaStream_t
 #define MUCA_CAT2(a, b) a##b
 #define MUCA_CAT(a, b) MUCA_CAT2(a, b)
 
-cudaError_t MUCA_CAT(launch_full_L, MUCA_L)(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s)
+cudaError_t MUCA_CAT(launch_full_L, MUCA_L)(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s)
 {
-    return ahead ? launch_full_t<MUCA_L, AttemptStream<MUCA_L, kTableStride>>(a, wpb, record, s)
-                 : launch_full_t<MUCA_L, DirectStream<MUCA_L, kTableStride>>(a, wpb, record, s);
+    if (form.chains > 0)
+        return launch_pair_t<MUCA_L>(a, form.chains, record, s);
+    return form.ahead ? launch_full_t<MUCA_L, AttemptStream<MUCA_L, kTableStride>>(a, wpb, record, s)
+                      : launch_full_t<MUCA_L, DirectStream<MUCA_L, kTableStride>>(a, wpb, record, s);
 }
 
 }  // namespace muca

@@ -2,6 +2,7 @@
 // device kernels (muca_kernels.cu and the other kernel files).  Not part of the public ABI.
 #pragma once
 
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 
@@ -89,6 +90,41 @@ __host__ __device__ inline RowPlan row_plan(int L, uint64_t t0, uint64_t n)
     return p;
 }
 
+// Largest dynamic shared memory a block may use on this device (bytes; 0 if the device does
+// not answer).
+size_t sweep_smem_limit();
+
+// Allows a kernel the device's whole shared memory, once per kernel and device: `done` has
+// a bit per device (the attribute is a bound only, and setting it takes microseconds).
+template <class Kernel>
+cudaError_t allow_smem(Kernel kern, std::atomic<uint64_t> &done)
+{
+    int dev = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess)
+        return err;
+    const uint64_t bit = dev < 64 ? 1ull << dev : 0ull;
+    if (done.load(std::memory_order_acquire) & bit)
+        return cudaSuccess;
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_smem_limit());
+    if (err == cudaSuccess)
+        done.fetch_or(bit, std::memory_order_release);
+    return err;
+}
+
+// Form of a sweep launch: `chains` > 0: paired kernel with that many chain warps per block
+// (muca_pair.cuh); else one thread per walker, the thresholds loaded two attempts ahead or
+// directly (muca_device.cuh).
+struct SweepForm {
+    int32_t chains;
+    bool ahead;
+};
+
+// Waits between the warps of the paired kernel: tries of at most 20 us each before a wait
+// gives up (a slot of the ring turns over in a few microseconds).
+constexpr uint32_t kPairWaitTries = 1u << 16;
+constexpr int kPairMaxThreads = 128;
+
 // Device state of an iteration whose recursion runs on the device (muca_iterate_device).
 struct IterState {
     uint32_t done;       // 0: running; 1: the last histogram was flat; 2: iteration limit
@@ -134,9 +170,6 @@ size_t sizing_smem_bytes(int L, int walkers_per_block);
 size_t full_smem_bytes(int L, int walkers_per_block, bool record, bool guard = false, int stride = kTableStride);
 size_t launch_smem_bytes(int L, int walkers_per_block, bool guard = false, int stride = kTableStride);
 
-// Largest dynamic shared memory a block may use on this device (bytes).
-size_t sweep_smem_limit();
-
 // Runs a.n_therm thermalization attempts from a.t0 (recording launches only; may be 0),
 // then a.n attempts of every walker: one launch unless the range crosses a step of counter
 // word 1 (every 2^34 attempts).  Grid = ceil(W / walkers_per_block).
@@ -164,24 +197,23 @@ cudaError_t launch_unpack(int32_t L, int32_t layout, int64_t W, const void *latt
 cudaError_t launch_philox(const uint32_t *ctr, uint32_t k0, uint32_t k1, size_t n, uint32_t *out,
                           cudaStream_t s);
 
-// Kernels of one L each (muca_full_L.cu): launch over any attempt range, with the
-// thresholds loaded two attempts ahead or directly.
-cudaError_t launch_full_L4(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s);
-cudaError_t launch_full_L8(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s);
-cudaError_t launch_full_L12(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s);
-cudaError_t launch_full_L16(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s);
-cudaError_t launch_full_L20(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s);
-cudaError_t launch_full_L24(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s);
-cudaError_t launch_full_L28(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s);
-cudaError_t launch_full_L32(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s);
-cudaError_t launch_full_L36(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s);
-cudaError_t launch_full_L40(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s);
-cudaError_t launch_full_L44(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s);
-cudaError_t launch_full_L48(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s);
-cudaError_t launch_full_L52(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s);
-cudaError_t launch_full_L56(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s);
-cudaError_t launch_full_L60(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s);
-cudaError_t launch_full_L64(const SweepArgs &a, int wpb, bool ahead, bool record, cudaStream_t s);
+// Kernels of one L each (muca_full_L.cu): launch over any attempt range in the given form.
+cudaError_t launch_full_L4(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
+cudaError_t launch_full_L8(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
+cudaError_t launch_full_L12(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
+cudaError_t launch_full_L16(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
+cudaError_t launch_full_L20(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
+cudaError_t launch_full_L24(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
+cudaError_t launch_full_L28(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
+cudaError_t launch_full_L32(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
+cudaError_t launch_full_L36(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
+cudaError_t launch_full_L40(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
+cudaError_t launch_full_L44(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
+cudaError_t launch_full_L48(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
+cudaError_t launch_full_L52(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
+cudaError_t launch_full_L56(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
+cudaError_t launch_full_L60(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
+cudaError_t launch_full_L64(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
 
 // Blocks of the sweep kernel for this L, layout and block size that one SM holds at once
 // by the sizing rule (0 if the configuration does not fit).

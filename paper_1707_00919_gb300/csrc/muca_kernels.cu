@@ -129,42 +129,43 @@ __global__ void philox_kernel(const uint32_t *ctr, uint32_t k0, uint32_t k1, siz
     out[4 * i + 3] = r.w;
 }
 
-// Whether a launch takes the attempt stream with the two-ahead loads: unless its SMs hold
-// more than two warps per sub-partition at once, which cover the direct loads' latency
-// (both sides measured at the line: muca_device.cuh, DirectStream).
-bool ahead_of_loads(const SweepArgs &a, int wpb)
+// The form of a launch by the warps of walkers per SM: up to two, the paired kernel (its
+// generator warps on the sub-partitions that would idle); up to eight, two per
+// sub-partition, the two-ahead loads; more than that resident at once, direct loads, whose
+// latency the other warps cover.
+SweepForm sweep_form(const SweepArgs &a, int wpb)
 {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-        return true;
+        return {0, true};
     const int64_t warps = (a.W + 31) / 32;
-    if (warps <= 8 * (int64_t)sms)
-        return true;
-    return resident_blocks(a.L, a.layout, wpb) * (wpb / 32) <= 8;
+    if (warps <= 2 * (int64_t)sms)
+        return {warps <= sms ? 1 : 2, true};
+    return {0, warps <= 8 * (int64_t)sms || resident_blocks(a.L, a.layout, wpb) * (wpb / 32) <= 8};
 }
 
 // Dispatches a launch to the kernel for L.
 cudaError_t launch_full(const SweepArgs &a, int wpb, bool record, cudaStream_t s)
 {
-    const bool ahead = ahead_of_loads(a, wpb);
+    const SweepForm form = sweep_form(a, wpb);
     switch (a.L) {
-    case 4: return launch_full_L4(a, wpb, ahead, record, s);
-    case 8: return launch_full_L8(a, wpb, ahead, record, s);
-    case 12: return launch_full_L12(a, wpb, ahead, record, s);
-    case 16: return launch_full_L16(a, wpb, ahead, record, s);
-    case 20: return launch_full_L20(a, wpb, ahead, record, s);
-    case 24: return launch_full_L24(a, wpb, ahead, record, s);
-    case 28: return launch_full_L28(a, wpb, ahead, record, s);
-    case 32: return launch_full_L32(a, wpb, ahead, record, s);
-    case 36: return launch_full_L36(a, wpb, ahead, record, s);
-    case 40: return launch_full_L40(a, wpb, ahead, record, s);
-    case 44: return launch_full_L44(a, wpb, ahead, record, s);
-    case 48: return launch_full_L48(a, wpb, ahead, record, s);
-    case 52: return launch_full_L52(a, wpb, ahead, record, s);
-    case 56: return launch_full_L56(a, wpb, ahead, record, s);
-    case 60: return launch_full_L60(a, wpb, ahead, record, s);
-    case 64: return launch_full_L64(a, wpb, ahead, record, s);
+    case 4: return launch_full_L4(a, wpb, form, record, s);
+    case 8: return launch_full_L8(a, wpb, form, record, s);
+    case 12: return launch_full_L12(a, wpb, form, record, s);
+    case 16: return launch_full_L16(a, wpb, form, record, s);
+    case 20: return launch_full_L20(a, wpb, form, record, s);
+    case 24: return launch_full_L24(a, wpb, form, record, s);
+    case 28: return launch_full_L28(a, wpb, form, record, s);
+    case 32: return launch_full_L32(a, wpb, form, record, s);
+    case 36: return launch_full_L36(a, wpb, form, record, s);
+    case 40: return launch_full_L40(a, wpb, form, record, s);
+    case 44: return launch_full_L44(a, wpb, form, record, s);
+    case 48: return launch_full_L48(a, wpb, form, record, s);
+    case 52: return launch_full_L52(a, wpb, form, record, s);
+    case 56: return launch_full_L56(a, wpb, form, record, s);
+    case 60: return launch_full_L60(a, wpb, form, record, s);
+    case 64: return launch_full_L64(a, wpb, form, record, s);
     default: return cudaErrorNotSupported;
     }
 }

@@ -393,11 +393,10 @@ cudaError_t launch_random_t(const SweepArgs &a, int wpb, cudaStream_t s)
     const size_t smem = random_smem_bytes_t<RowT>(a.L, wpb, RECORD);
     auto kern = a.L == 8 * (int)sizeof(RowT) ? random_sweep_kernel<RowT, LAYOUT, RECORD, true>
                                               : random_sweep_kernel<RowT, LAYOUT, RECORD, false>;
-    if (smem > 48 * 1024) {
-        const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (err != cudaSuccess)
-            return err;
-    }
+    static std::atomic<uint64_t> allowed[2];
+    const cudaError_t err = allow_smem(kern, allowed[a.L == 8 * (int)sizeof(RowT) ? 0 : 1]);
+    if (err != cudaSuccess)
+        return err;
     const int64_t blocks = (a.W + wpb - 1) / wpb;
     kern<<<(unsigned)blocks, wpb, smem, s>>>(a);
     return cudaGetLastError();

@@ -46,6 +46,40 @@ def test_every_size_and_cut(M, orc, L):
         assert np.array_equal(m.get_lattice(), s)
 
 
+@pytest.mark.parametrize("L", [4, 8, 12, 24, 28, 32, 48, 60, 64])
+@pytest.mark.parametrize("warps_per_sm", [0, 1, 2])
+def test_forms_by_walker_count(M, orc, L, warps_per_sm):
+    """One and two chain warps per block with their generators, one thread per walker with
+    the loads two attempts ahead; a fused launch cut at both ends, then unrecorded rows and a
+    recorded part of a row, a ragged last warp."""
+    import torch
+    W = torch.cuda.get_device_properties(0).multi_processor_count * 32 * warps_per_sm + 77
+    seed, N = 11, L * L
+    lnW = rand_weights(L, 3 * L)
+    T = orc.build_table(L, lnW)
+    therm, rec, more, last = 3 * L + 6, 2 * L + 3, 5 * L + 1, L // 2
+    with M.Muca(L, W, seed, layout=warps_per_sm % 2) as m:
+        m.set_weights(lnW)
+        m.set_attempt_counter(5)
+        m.thermalize_and_record(therm, rec)
+        m.attempts(more, False)
+        m.attempts(last, True)
+        H, e, lat = m.get_histogram(), m.get_energies(), m.get_lattice()
+    assert int(H.sum()) == W * (rec + last)
+    Ho = np.zeros(N + 1, dtype=np.uint64)
+    whole = L <= 12 or warps_per_sm == 0
+    for w0, n in ([(0, W)] if whole else [(0, 64), (W - 77, 77)]):
+        s, eo = orc.init(L, seed, n, walker0=w0)
+        orc.run(L, seed, s, eo, T, 5, therm, False, walker0=w0)
+        orc.run(L, seed, s, eo, T, 5 + therm, rec, True, Ho, walker0=w0)
+        orc.run(L, seed, s, eo, T, 5 + therm + rec, more, False, walker0=w0)
+        orc.run(L, seed, s, eo, T, 5 + therm + rec + more, last, True, Ho, walker0=w0)
+        assert np.array_equal(lat[w0:w0 + n], s)
+        assert np.array_equal(e[w0:w0 + n], eo)
+    if whole:
+        assert np.array_equal(H, Ho)
+
+
 @pytest.mark.parametrize("L,extra", [(8, 0), (8, 45), (12, 45), (20, 31), (32, 45)])
 def test_many_warps(M, orc, L, extra):
     """More than two warps per SM sub-partition: the form with direct loads."""
