@@ -179,7 +179,6 @@ cudaError_t launch_sweep(const SweepArgs &a, int walkers_per_block, bool record,
 // any L, any attempt range; the given block size, or a smaller one that fits shared
 // memory).
 cudaError_t launch_random_sweep(const SweepArgs &a, int walkers_per_block, bool record, cudaStream_t s);
-size_t random_smem_bytes(int L, int walkers_per_block, bool record);
 
 // Draws the initial spins (tag 1 stream) and their energy indices.
 cudaError_t launch_init(int32_t L, int32_t layout, int64_t W, uint64_t seed, uint32_t walker0, void *lattice,

@@ -104,6 +104,28 @@ def test_many_warps(M, orc, L, extra):
             assert np.array_equal(H, Ho)
 
 
+@pytest.mark.parametrize("L", range(4, 65, 4))
+def test_random_order_every_size(M, orc, L):
+    """Windows cut by conflicts, chunks of sites, heads and tails inside a Philox block."""
+    W, seed, N = 77, 21 + L, L * L
+    lnW = rand_weights(L, 5 * L)
+    T = orc.build_table(L, lnW)
+    s, e = orc.init(L, seed, W)
+    t = 0
+    with M.Muca(L, W, seed, layout=(L // 4) % 2) as m:
+        m.set_weights(lnW)
+        m.site_order = M.MUCA_ORDER_RANDOM
+        for n, rec in [(1, True), (1, False), (9, True), (4, True), (510, True), (1026, False), (700, True)]:
+            m.reset_histogram()
+            m.attempts(n, rec)
+            Ho = orc.run(L, seed, s, e, T, t, n, rec, site_order=1)
+            t += n
+            if rec:
+                assert np.array_equal(m.get_histogram(), Ho)
+            assert np.array_equal(m.get_energies(), e)
+        assert np.array_equal(m.get_lattice(), s)
+
+
 def test_batch_across_counter_word(M):
     """Ranges that cross t = 2^34 inside a batched launch equal the instances run alone."""
     specs = [(8, 70), (24, 33), (64, 40)]
