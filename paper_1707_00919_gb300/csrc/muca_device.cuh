@@ -393,7 +393,7 @@ __device__ __forceinline__ uint32_t left_of(const uint32_t (&C)[row_words(L)], i
 // dp4a (a four-byte dot product) adds a constant multiple of one site's count to an
 // address: one instruction on the multiply pipe where a shift, a mask and an addition
 // took three on the integer ALU, the pipe with the most instructions of this loop.
-template <int L>
+template <int L, bool SHIFTED = false>
 struct RowCounts {
     static constexpr int NW = row_words(L);
     uint32_t k0[2 * NW];   // if the left neighbour did not flip
@@ -401,10 +401,14 @@ struct RowCounts {
 
     __device__ __forceinline__ RowCounts(const uint32_t (&U)[NW], const uint32_t (&C)[NW], const uint32_t (&D)[NW])
     {
+        uint32_t hr[NW];   // right disagreements; shifted by a site they are the left ones
+#pragma unroll
+        for (int i = 0; i < NW; ++i)
+            hr[i] = C[i] ^ right_of<L>(C, i);
 #pragma unroll
         for (int i = 0; i < NW; ++i) {
-            const uint32_t kb = (U[i] ^ C[i]) + (D[i] ^ C[i]) + (C[i] ^ right_of<L>(C, i));
-            const uint32_t h0 = C[i] ^ left_of<L>(C, i);
+            const uint32_t kb = (U[i] ^ C[i]) + (D[i] ^ C[i]) + hr[i];
+            const uint32_t h0 = SHIFTED ? left_of<L>(hr, i) : C[i] ^ left_of<L>(C, i);
             const uint32_t a = kb + h0, b = kb + 0x11111111u - h0;
             k0[2 * i] = a & 0x0F0F0F0Fu;
             k0[2 * i + 1] = (a >> 4) & 0x0F0F0F0Fu;
@@ -429,6 +433,14 @@ struct RowCounts {
     }
 };
 
+// w with the bit flipped if acc: one predicated instruction instead of a select and an
+// exclusive-or.
+__device__ __forceinline__ uint32_t flip_if(uint32_t w, uint32_t bit, bool acc)
+{
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p xor.b32 %0, %0, %2;\n\t}" : "+r"(w) : "r"(acc ? 1u : 0u), "r"(bit));
+    return w;
+}
+
 // acc + m * (count of site x in its count word w), m in [-128, 127].
 __device__ __forceinline__ uint32_t add_count(uint32_t w, int x, int m, uint32_t acc)
 {
@@ -447,13 +459,24 @@ __device__ __forceinline__ uint32_t add_count(uint32_t w, int x, int m, uint32_t
 // What bounds it: instruction issue.  A warp alone on its SM sub-partition issues one
 // half-rate instruction per two cycles whatever its pipe (a wide multiply takes four), so
 // at one warp the attempt costs twice its ALU and multiply instructions; with two warps
-// the pipes overlap in part.  Measured at L = 32, 16384 walkers: 27.2 instructions per
-// attempt (13.5 ALU, 8.7 multiply pipe, of them 4 wide, 3.1 LSU) against 31.1 with shifted
-// and masked fields, 24.9 us per sweep against 25.6 (one warp per sub-partition); 62.2
-// against 67.8 us at 48 640 walkers; L = 64, 32 768 walkers 169 against 186 us.
+// the pipes overlap in part.  A chain warp whose words come from other warps (muca_pair.cuh)
+// has half the instructions and is bound by the latency of its chain instead.  EARLY says
+// how much is formed for both outcomes before a decision and selected by it: 0 nothing,
+// 1 the row address if the next attempt flips, 2 also the address of its flipped candidate:
+// each step shortens the chain and adds instructions.  The histogram's reduction comes
+// after the loads, which it would delay.  Measured, us per sweep (EARLY 0 / 1 / 2):
+//   L = 32, 16 384 walkers, one warp per sub-partition      24.7 / 24.4 / 24.4
+//   L = 32, 38 912 walkers, two warps                       41.9 / 42.0 / 43.1
+//   L = 64, 32 768 walkers, 1.75 warps                      166  / 169  / 177
+//   L = 32, 4096 walkers, chain warps with generators       18.7 / 18.2 / 17.7
+//   L = 64, 4096 walkers, the same                          74.8 / 74.2 / 72.1
+//   L = 8, 128 walkers, the same                            1.23 / 1.16 / 1.28
+// (24.9 at 16 384 walkers with selects and exclusive-ors for the flips and the reduction
+// first; 25.6 with shifted and masked count fields, 31.1 instructions per attempt.)
 // ---------------------------------------------------------------------------------
-template <int L, int STRIDE>
+template <int L, int STRIDE, int EARLY>
 struct AttemptStream {
+    using Counts = RowCounts<L, EARLY == 0 && (L > 32)>;
     static constexpr int NW = row_words(L);
     static constexpr int kStep = -4 * STRIDE;          // row step of a flip: 4 STRIDE (2 - k) bytes
     static constexpr uint32_t kTwo = 8u * STRIDE;
@@ -466,7 +489,7 @@ struct AttemptStream {
     __device__ __forceinline__ void start(const uint32_t (&U)[NW], const uint32_t (&C)[NW], const uint32_t (&D)[NW],
                                           uint32_t E0)
     {
-        const RowCounts<L> k(U, C, D);
+        const Counts k(U, C, D);
         E = E0;
         prev_acc = false;
         Eacc = add_count(k.word0(0), 0, kStep, E0 + kTwo);
@@ -481,9 +504,9 @@ struct AttemptStream {
     __device__ __forceinline__ void row(const uint32_t (&U)[NW], uint32_t (&C)[NW], const uint32_t (&D)[NW],
                                         const uint32_t (&D2)[NW], Src &src)
     {
-        RowCounts<L> k(U, C, D);
+        Counts k(U, C, D);
         uint32_t n0e = 0u, n0o = 0u, n1o = 0u;   // counts of the next row's sites 0 (n0e) and 1 (n0o, n1o)
-        const uint32_t adj_if_flip = RowCounts<L>::last_step(C);
+        const uint32_t adj_if_flip = Counts::last_step(C);
 #pragma unroll
         for (int xb = 0; xb < L; xb += 4) {
             const uint4 rw = src.get(xb);
@@ -493,13 +516,27 @@ struct AttemptStream {
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int x = xb + u;
+                // counts for the step of attempt x + 1 (0: if x stays, 1: if it flips) and for the
+                // candidates of attempt x + 2, in this row or the next (site 0's left neighbour
+                // comes later)
+                const uint32_t s0 = x + 1 == L ? n0e : k.word0(x + 1), s1 = x + 1 == L ? n0e : k.word1(x + 1);
+                const uint32_t j0 = x + 2 < L ? k.word0(x + 2) : x + 2 == L ? n0e : n0o;
+                const uint32_t j1 = x + 2 < L ? k.word1(x + 2) : x + 2 == L ? n0e : n1o;
+                uint32_t stay = 0u, move = 0u, at_stay = 0u, at_move = 0u;
+                if (EARLY >= 1) {
+                    stay = add_count(s0, (x + 1) % L, kStep, E + kTwo);
+                    move = add_count(s1, (x + 1) % L, kStep, Eacc + kTwo);
+                }
+                if (EARLY >= 2) {
+                    at_stay = add_count(j1, (x + 2) % L, 4, stay);
+                    at_move = add_count(j1, (x + 2) % L, 4, move);
+                }
                 const uint32_t T = prev_acc ? T1n : T0n;
                 const bool acc = words[u] < T;
                 E = acc ? Eacc : E;
-                C[x >> 3] ^= acc ? (1u << (4 * (x & 7))) : 0u;
+                C[x >> 3] = flip_if(C[x >> 3], 1u << (4 * (x & 7)), acc);
                 if (x == 0)
                     k.add_to_last(acc ? adj_if_flip : 0u);
-                hist_add_one(E);
                 if (x == (L > 4 ? L - 5 : L - 3)) {
                     // the current row's sites 0 and 1 are final: the next row's first counts
                     const uint32_t kb = (C[0] ^ D[0]) + (D2[0] ^ D[0]) + (D[0] ^ right_of<L>(D, 0));
@@ -508,16 +545,18 @@ struct AttemptStream {
                     n0o = ((kb + h0) >> 4) & 0x0Fu;
                     n1o = ((kb + 0x11111111u - h0) >> 4) & 0x0Fu;
                 }
-                // row address if attempt x + 1 flips, candidates of attempt x + 2 (in this row
-                // or the next) for both its outcomes; site 0's left neighbour comes later
-                const uint32_t s = x + 1 == L ? n0e : acc ? k.word1(x + 1) : k.word0(x + 1);
-                const uint32_t j0 = x + 2 < L ? k.word0(x + 2) : x + 2 == L ? n0e : n0o;
-                const uint32_t j1 = x + 2 < L ? k.word1(x + 2) : x + 2 == L ? n0e : n1o;
-                Eacc = add_count(s, (x + 1) % L, kStep, E + kTwo);
+                if (EARLY >= 1)
+                    Eacc = acc ? move : stay;
+                else
+                    Eacc = add_count(acc ? s1 : s0, (x + 1) % L, kStep, E + kTwo);
                 T0n = T0nn;
                 T1n = T1nn;
                 T0nn = lds_u32(add_count(j0, (x + 2) % L, 4, E));
-                T1nn = lds_u32(add_count(j1, (x + 2) % L, 4, Eacc));
+                if (EARLY >= 2)
+                    T1nn = lds_u32(acc ? at_move : at_stay);
+                else
+                    T1nn = lds_u32(add_count(j1, (x + 2) % L, 4, Eacc));
+                hist_add_one(E);
                 prev_acc = acc;
             }
         }
@@ -874,7 +913,7 @@ __device__ __forceinline__ void sweep_block(const SweepArgs &a, const Plans &pla
 template <int L, bool GUARD = false, int STRIDE = kTableStride>
 __device__ __noinline__ void batch_item(const SweepArgs &a, const BatchItem &it, unsigned char *smem, bool record)
 {
-    sweep_block<L, GUARD, STRIDE, AttemptStream<L, STRIDE>>(a, DevicePlans{}, it.wbase, it.wpb, smem, record);
+    sweep_block<L, GUARD, STRIDE, AttemptStream<L, STRIDE, 0>>(a, DevicePlans{}, it.wbase, it.wpb, smem, record);
 }
 
 }  // namespace

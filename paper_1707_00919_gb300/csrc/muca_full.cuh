@@ -47,7 +47,7 @@ cudaError_t MUCA_CAT(launch_full_L, MUCA_L)(const SweepArgs &a, int wpb, SweepFo
 {
     if (form.chains > 0)
         return launch_pair_t<MUCA_L>(a, form.chains, record, s);
-    return form.ahead ? launch_full_t<MUCA_L, AttemptStream<MUCA_L, kTableStride>>(a, wpb, record, s)
+    return form.ahead ? launch_full_t<MUCA_L, AttemptStream<MUCA_L, kTableStride, (MUCA_L <= 32 ? 1 : 0)>>(a, wpb, record, s)
                       : launch_full_t<MUCA_L, DirectStream<MUCA_L, kTableStride>>(a, wpb, record, s);
 }
 

@@ -150,7 +150,7 @@ __device__ __forceinline__ uint32_t ring_rows(const SmemRows<L> &rows, uint32_t 
     rows.load(y == 0 ? L - 1 : y - 1, U);
     rows.load(y, C);
     rows.load(y + 1 == L ? 0 : y + 1, D);
-    AttemptStream<L, STRIDE> st;
+    AttemptStream<L, STRIDE, (L > 8 ? 2 : 1)> st;
     st.start(U, C, D, E);
 #pragma unroll 1
     for (uint64_t left = nrows; left > 0;) {
