@@ -94,11 +94,80 @@ int check_device_error(muca_t h)
     return MUCA_OK;
 }
 
+namespace {
+
+std::mutex g_queued_mutex;
+std::vector<muca_t> g_queued;   // instances with sweeps that the host has not waited for
+
+// Whether the instance's own stream has run dry.  A stream given by the caller is not
+// asked (the caller may have destroyed it): such an instance counts until it is waited for.
+// The query must not disturb a capture that another thread has under way.
+bool ran_dry(muca_t h)
+{
+    if (h->stream != h->own_stream)
+        return false;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess)
+        return false;
+    const cudaError_t err = cudaStreamQuery(h->stream);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (err != cudaSuccess)
+        cudaGetLastError();   // not ready is not an error of the launches to come
+    return err == cudaSuccess;
+}
+
+}  // namespace
+
+bool sweeps_queued(muca_t h)
+{
+    constexpr int kRemembered = 8;   // launches for which an overlap is taken to recur
+    std::lock_guard<std::mutex> lock(g_queued_mutex);
+    bool alone = true;
+    if (h->company > 0) {   // no query (microseconds) while the overlaps go on
+        --h->company;
+        alone = false;
+    }
+    bool listed = false;
+    for (size_t i = 0; i < g_queued.size(); ++i) {
+        const muca_t o = g_queued[i];
+        if (o == h) {
+            listed = true;
+        } else if (o->device == h->device) {
+            if (alone && ran_dry(o)) {
+                g_queued.erase(g_queued.begin() + (std::ptrdiff_t)i--);
+                continue;
+            }
+            if (alone)
+                h->company = kRemembered;
+            o->company = kRemembered;
+            alone = false;
+            break;   // the first one in flight is enough, and it is told
+        }
+    }
+    if (!listed && std::find(g_queued.begin(), g_queued.end(), h) == g_queued.end())
+        g_queued.push_back(h);
+    return alone;
+}
+
+void sweeps_waited(muca_t h)
+{
+    std::lock_guard<std::mutex> lock(g_queued_mutex);
+    g_queued.erase(std::remove(g_queued.begin(), g_queued.end(), h), g_queued.end());
+}
+
+cudaError_t wait_stream(muca_t h)
+{
+    const cudaError_t err = cudaStreamSynchronize(h->stream);
+    if (err == cudaSuccess)
+        sweeps_waited(h);
+    return err;
+}
+
 int sync_and_check(muca_t h)
 {
     MUCA_CUDA(cudaMemcpyAsync(h->h_err, h->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, h->stream),
               "error word read");
-    MUCA_CUDA(cudaStreamSynchronize(h->stream), "stream synchronize");
+    MUCA_CUDA(wait_stream(h), "stream synchronize");
     return check_device_error(h);
 }
 
@@ -124,13 +193,16 @@ static muca::SweepArgs sweep_args(muca_t h, uint64_t n, const uint32_t *skip)
 int run_attempts(muca_t h, uint64_t n, bool record, const uint32_t *skip)
 {
     const uint64_t cap = record ? max_recorded_attempts(h->wpb) : UINT64_MAX;
+    if (n == 0)
+        return MUCA_OK;
+    const bool alone = sweeps_queued(h);
     while (n > 0) {
         const uint64_t chunk = std::min(n, cap);
         const muca::SweepArgs a = sweep_args(h, chunk, skip);
         if (h->order == MUCA_ORDER_RANDOM)
             MUCA_CUDA(muca::launch_random_sweep(a, h->wpb, record, h->stream), "random-order sweep launch");
         else
-            MUCA_CUDA(muca::launch_sweep(a, h->wpb, record, h->stream), "sweep launch");
+            MUCA_CUDA(muca::launch_sweep(a, h->wpb, alone, record, h->stream), "sweep launch");
         h->t += chunk;
         n -= chunk;
     }
@@ -146,7 +218,7 @@ int run_therm_record(muca_t h, uint64_t n_therm, uint64_t n_record, const uint32
     }
     muca::SweepArgs a = sweep_args(h, n_record, skip);
     a.n_therm = n_therm;
-    MUCA_CUDA(muca::launch_sweep(a, h->wpb, true, h->stream), "sweep launch");
+    MUCA_CUDA(muca::launch_sweep(a, h->wpb, sweeps_queued(h), true, h->stream), "sweep launch");
     h->t += n_therm + n_record;
     return MUCA_OK;
 }
@@ -451,6 +523,9 @@ int muca_create_ex(const muca_options *opt, muca_t *out)
     if (err != cudaSuccess)
         return cleanup(cuda_fail(err, "stream create"));
     h->stream = h->own_stream;
+    err = cudaGetDevice(&h->device);
+    if (err != cudaSuccess)
+        return cleanup(cuda_fail(err, "device query"));
     err = cudaEventCreateWithFlags(&h->table_copied, cudaEventDisableTiming);
     if (err != cudaSuccess)
         return cleanup(cuda_fail(err, "event create"));
@@ -499,6 +574,7 @@ int muca_destroy(muca_t h)
         return MUCA_OK;
     if (h->stream)
         cudaStreamSynchronize(h->stream);
+    sweeps_waited(h);
     device_free(h->alloc, h->block);
     device_free(h->alloc, h->iter_block);
     if (h->h_iter)
@@ -578,7 +654,7 @@ int muca_set_stream(muca_t h, void *cuda_stream)
     int rc = validate(h);
     if (rc)
         return rc;
-    MUCA_CUDA(cudaStreamSynchronize(h->stream), "stream synchronize");
+    MUCA_CUDA(wait_stream(h), "stream synchronize");
     h->stream = cuda_stream ? static_cast<cudaStream_t>(cuda_stream) : h->own_stream;
     return MUCA_OK;
 }
@@ -617,7 +693,7 @@ int muca_get_table(muca_t h, uint32_t *T_out, size_t n)
         return fail(MUCA_EINVAL, "table has %d entries", (h->N + 1) * 5);
     MUCA_CUDA(cudaMemcpyAsync(T_out, h->d_table, n * sizeof(uint32_t), cudaMemcpyDeviceToHost, h->stream),
               "table read");
-    MUCA_CUDA(cudaStreamSynchronize(h->stream), "stream synchronize");
+    MUCA_CUDA(wait_stream(h), "stream synchronize");
     return MUCA_OK;
 }
 
@@ -699,7 +775,7 @@ int muca_get_lattice(muca_t h, int8_t *out, size_t n)
     if (err == cudaSuccess)
         err = cudaMemcpyAsync(out, tmp, total, cudaMemcpyDeviceToHost, h->stream);
     // the buffer goes back to the allocator only after every use of it has finished
-    const cudaError_t sync = cudaStreamSynchronize(h->stream);
+    const cudaError_t sync = wait_stream(h);
     if (err == cudaSuccess)
         err = sync;
     device_free(h->alloc, tmp);
@@ -725,7 +801,7 @@ int muca_set_lattice(muca_t h, const int8_t *spins, size_t n)
     cudaError_t err = cudaMemcpyAsync(tmp, spins, total, cudaMemcpyHostToDevice, h->stream);
     if (err == cudaSuccess)
         err = muca::launch_pack(h->L, h->layout, h->W, tmp, h->d_lattice, h->d_energy, h->stream);
-    const cudaError_t sync = cudaStreamSynchronize(h->stream);
+    const cudaError_t sync = wait_stream(h);
     if (err == cudaSuccess)
         err = sync;
     device_free(h->alloc, tmp);
@@ -854,7 +930,7 @@ int muca_load(const char *path, muca_t *out)
     cudaError_t err = cudaMemcpyAsync(h->d_hist, h->h_hist, nb * sizeof(unsigned long long), cudaMemcpyHostToDevice,
                                       h->stream);
     if (err == cudaSuccess)
-        err = cudaStreamSynchronize(h->stream);
+        err = wait_stream(h);
     if (err != cudaSuccess)
         return cleanup(cuda_fail(err, "histogram upload"));
     h->t = t;

@@ -454,7 +454,7 @@ int muca_batch_create(const muca_t *instances, int32_t n, muca_batch_t *out)
         return cleanup(cuda_fail(err, "batch pinned buffers"));
     // from now on every call on a member instance is ordered with the batch's work
     for (muca_t h : b->inst) {
-        err = cudaStreamSynchronize(h->stream);
+        err = wait_stream(h);
         if (err != cudaSuccess)
             return cleanup(cuda_fail(err, "instance synchronize"));
         b->saved_streams.push_back(h->stream);

@@ -313,7 +313,7 @@ int muca_iterate_device(muca_t h, const muca_params *p_in, int32_t iterations_pe
     const uint64_t n_therm = p.therm_sweeps * (uint64_t)N, n_upd = p.sweeps_per_iter * (uint64_t)N;
     const uint64_t t_start = h->t;
     // the first table and the weights from the host; the state zeroed
-    MUCA_CUDA(cudaStreamSynchronize(h->stream), "stream synchronize");
+    MUCA_CUDA(wait_stream(h), "stream synchronize");
     std::memset(h->h_iter, 0, sizeof(muca::IterState));
     h->h_iter->prev_lo = p.resume ? h->sched.prev_lo : -1;
     h->h_iter->prev_hi = p.resume ? h->sched.prev_hi : -1;
@@ -355,7 +355,7 @@ int muca_iterate_device(muca_t h, const muca_params *p_in, int32_t iterations_pe
     h->t = t_start + (uint64_t)st.iterations * (n_therm + n_upd);
     MUCA_CUDA(cudaMemcpyAsync(h->lnW.data(), h->d_lnW, nb * sizeof(double), cudaMemcpyDeviceToHost, h->stream),
               "weights read");
-    MUCA_CUDA(cudaStreamSynchronize(h->stream), "stream synchronize");
+    MUCA_CUDA(wait_stream(h), "stream synchronize");
     const bool flat = st.done == 1u;
     if (st.iterations > (flat ? 1 : 0)) {   // at least one weight update: the state the host loop keeps
         h->sched.prev_lo = st.prev_lo;

@@ -61,6 +61,8 @@ struct muca_s {
     uint64_t seed = 0;
     int32_t layout = MUCA_LAYOUT_INT8;
     int32_t wpb = 64;
+    int device = 0;
+    int company = 0;                 // launches for which its sweeps are taken to overlap others (sweeps_queued)
     muca_host::Allocator alloc;
     cudaStream_t own_stream = nullptr;
     cudaStream_t stream = nullptr;
@@ -99,6 +101,16 @@ void build_table(int32_t L, const std::vector<double> &lnW, uint32_t *T);
 int upload_table(muca_t h);
 int check_device_error(muca_t h);
 int sync_and_check(muca_t h);
+// Which instances have sweeps that the host has not waited for, so that a launch knows
+// whether it has the device to itself (launch_sweep's form; results do not depend on it).
+// sweeps_queued notes that h is about to launch one and returns true if no other instance
+// of the device has one in flight, or had one together with h in the last few launches (who
+// queues several instances in turn does so again); sweeps_waited notes that h's stream has
+// been waited for.
+bool sweeps_queued(muca_t h);
+void sweeps_waited(muca_t h);
+// Waits for the instance's stream.
+cudaError_t wait_stream(muca_t h);
 int run_attempts(muca_t h, uint64_t n, bool record, const uint32_t *skip = nullptr);
 // n_therm attempts without recording, then n_record recorded ones (the histogram is not
 // zeroed here); one kernel launch where the whole-sweep kernel allows it.

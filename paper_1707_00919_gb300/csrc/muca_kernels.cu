@@ -129,26 +129,33 @@ __global__ void philox_kernel(const uint32_t *ctr, uint32_t k0, uint32_t k1, siz
     out[4 * i + 3] = r.w;
 }
 
-// The form of a launch by the warps of walkers per SM: up to two, the paired kernel (its
-// generator warps on the sub-partitions that would idle); up to eight, two per
-// sub-partition, the two-ahead loads; more than that resident at once, direct loads, whose
-// latency the other warps cover.
-SweepForm sweep_form(const SweepArgs &a, int wpb)
+// The form of a launch by the warps of walkers per SM.  Up to two, and with the device to
+// itself: the paired kernel, its generator warps on the sub-partitions that would idle
+// (when sweeps of other instances run, it would take SMs from them for less throughput:
+// eight instances of L = 32 with 4096 walkers, all queued, 1661 us per 20 sweeps with it
+// against 955).  Up to eight, two per sub-partition: the two-ahead loads.  More than that
+// resident at once: direct loads, whose latency the other warps cover.
+SweepForm sweep_form(const SweepArgs &a, int wpb, bool alone)
 {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
         return {0, true};
     const int64_t warps = (a.W + 31) / 32;
-    if (warps <= 2 * (int64_t)sms)
-        return {warps <= sms ? 1 : 2, true};
+    if (alone && warps <= 2 * (int64_t)sms) {
+        // one chain warp per block spreads them over the SMs; from L = 52 on the table leaves
+        // room for one block per SM only, and two chains share it, so that a sweep queued
+        // after this one finds SMs
+        const bool two = warps > sms || (a.L >= 52 && warps > 1);
+        return {two ? 2 : 1, true};
+    }
     return {0, warps <= 8 * (int64_t)sms || resident_blocks(a.L, a.layout, wpb) * (wpb / 32) <= 8};
 }
 
 // Dispatches a launch to the kernel for L.
-cudaError_t launch_full(const SweepArgs &a, int wpb, bool record, cudaStream_t s)
+cudaError_t launch_full(const SweepArgs &a, int wpb, bool alone, bool record, cudaStream_t s)
 {
-    const SweepForm form = sweep_form(a, wpb);
+    const SweepForm form = sweep_form(a, wpb, alone);
     switch (a.L) {
     case 4: return launch_full_L4(a, wpb, form, record, s);
     case 8: return launch_full_L8(a, wpb, form, record, s);
@@ -203,7 +210,7 @@ size_t sweep_smem_limit()
     return (size_t)v;
 }
 
-cudaError_t launch_sweep(const SweepArgs &a, int wpb, bool record, cudaStream_t s)
+cudaError_t launch_sweep(const SweepArgs &a, int wpb, bool alone, bool record, cudaStream_t s)
 {
     if (a.W == 0 || (a.n == 0 && a.n_therm == 0))
         return cudaSuccess;
@@ -212,16 +219,16 @@ cudaError_t launch_sweep(const SweepArgs &a, int wpb, bool record, cudaStream_t 
         // not one launch: the thermalization by itself
         part.n_therm = 0;
         part.n = a.n_therm;
-        const cudaError_t err = launch_sweep(part, wpb, false, s);
+        const cudaError_t err = launch_sweep(part, wpb, alone, false, s);
         if (err != cudaSuccess)
             return err;
         part.t0 = a.t0 + a.n_therm;
         part.n = a.n;
-        return launch_sweep(part, wpb, record, s);
+        return launch_sweep(part, wpb, alone, record, s);
     }
     for (uint64_t left = a.n; left > 0; left -= part.n, part.t0 += part.n) {
         part.n = a.n_therm > 0 ? left : same_word1(part.t0, left);
-        const cudaError_t err = launch_full(part, wpb, record, s);
+        const cudaError_t err = launch_full(part, wpb, alone, record, s);
         if (err != cudaSuccess)
             return err;
     }
