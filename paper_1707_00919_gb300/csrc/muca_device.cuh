@@ -752,39 +752,46 @@ struct DevicePlans {
 };
 
 // The thresholds into the block's table rows as asynchronous 4-byte copies (the caller
-// waits for them before its barrier), every other word of the NR rows zeroed; row G holds
-// energy 0.
+// waits for them before its barrier), the counts zeroed, and the thresholds of the rows
+// outside energies 0..N (row G holds energy 0).  A thread takes whole rows: no division per
+// word, which made this loop 9 us of a launch at L = 64.  It is not unrolled: that changed
+// the compiler's schedule of the attempts far below it (L = 32, 16384 walkers: 25.5 us per
+// sweep instead of 24.5).
 template <int NB, int NR, int G, int STRIDE>
 __device__ __forceinline__ void load_table(uint32_t *sTab, const uint32_t *table, int tid, int nthr)
 {
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(sTab);
-    for (int i = tid; i < NB * 5; i += nthr) {
-        const int e = i / 5, k = i - e * 5;
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sbase + 4u * (uint32_t)((e + G) * STRIDE + k)),
-                     "l"(table + i)
-                     : "memory");
+#pragma unroll 1
+    for (int e = tid; e < NB; e += nthr) {
+        const uint32_t at = sbase + (uint32_t)((e + G) * (4 * STRIDE));
+#pragma unroll
+        for (int k = 0; k < 5; ++k)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(at + 4u * k), "l"(table + e * 5 + k) : "memory");
+        sTab[(e + G) * STRIDE + kHistSlot] = 0u;
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
-    for (int i = tid; i < NR * STRIDE; i += nthr) {
-        const int r = i / STRIDE, k = i - r * STRIDE;
-        if (k >= 5 || r < G || r >= G + NB)
-            sTab[i] = 0u;
+    for (int i = tid; i < (NR - NB) * STRIDE; i += nthr) {
+        const int r = i / STRIDE;
+        sTab[(r < G ? r : r + NB) * STRIDE + (i - r * STRIDE)] = 0u;
     }
 }
 
 // A walker's lattice (warp-cooperatively where the warp is full) into shared memory, and
 // back.  Every lane of the warp calls them; lanes without a walker get an empty lattice.
-template <int L>
+// Bound by latency: few warps run, so each keeps many loads in flight - 16 packed rows, RB
+// rows of bytes, a whole row of a ragged walker count (L = 64, 9000 walkers of bytes: what a
+// launch takes besides its sweeps went from 174 to 87 us; 16384 packed ones, 36 to 23).
+template <int L, int RB = 4>
 __device__ __forceinline__ void load_lattice(const SweepArgs &a, const SmemRows<L> &rows, int64_t w, bool active,
                                              bool warp_full, int lane)
 {
     using RowT = typename RowOf<L>::type;
     if (a.layout == MUCA_LAYOUT_PACKED) {
-#pragma unroll 4
+#pragma unroll 16
         for (int y = 0; y < L; ++y)
             rows.store_bits(y, active ? reinterpret_cast<const RowT *>(a.lattice)[(size_t)y * a.W + w] : (RowT)0);
     } else if (warp_full) {
-        constexpr int RB = 4;   // rows per batch of loads
+        // RB rows per batch of loads
         for (int y = 0; y < L; y += RB) {
             RowT r[RB];
             warp_load_rows_int8<L, RB, RowT>(reinterpret_cast<const int8_t *>(a.lattice), a.W, w - lane, y, lane, r);
@@ -797,7 +804,7 @@ __device__ __forceinline__ void load_lattice(const SweepArgs &a, const SmemRows<
         for (int y = 0; y < L; ++y) {
             RowT r = 0;
             if (active) {
-#pragma unroll 16
+#pragma unroll
                 for (int x = 0; x < L; ++x)   // unrolled: a row's loads are in flight together
                     r |= (RowT)(g[(size_t)(y * L + x) * a.W + w] < 0) << x;
             }

@@ -215,7 +215,10 @@ __global__ void __launch_bounds__(kPairMaxThreads, 1) pair_kernel(const SweepArg
     load_table<NB, NB + 1, 0, STRIDE>(sTab, a.table, tid, nthr);
     int32_t e = 0;
     if (chain && pair_on) {
-        load_lattice<L>(a, rows, w, active, warp_full, lane);
+        // Eight rows in flight: one warp per SM has only its own loads to hide their latency
+        // behind, and in this kernel the registers are free (L = 48, 1024 walkers, spins as
+        // bytes: 45 us of a launch that are not sweeps with four, 32 with eight).
+        load_lattice<L, (L % 8 == 0 ? 8 : 4)>(a, rows, w, active, warp_full, lane);
         if (active) {
             e = a.energy[w];
             if (e < 0 || e > N) {
