@@ -14,34 +14,58 @@ namespace {
 // Initial spins: +1 iff the top bit of the tag-1 word for attempt number t = site is
 // clear; the energy index is the number of unsatisfied bonds over two.
 // ---------------------------------------------------------------------------------
+// Blocks of 32 walkers, one lane each, and a warp per strip of kStrip rows.  One thread per
+// walker and all its rows left most of the device idle and the strips' latency in series:
+// a lattice of L = 64 and 8106 walkers (33 MB) took 148 us to make and 360 us to take over from
+// the host's format, in strips 53 and 52.
+constexpr int kStrip = 4;
+constexpr int kMaxStrips = 64 / kStrip;
+
 // Writes a walker's lattice, given row by row (bit x = spin at x is down), in the
 // instance's layout, and its energy index: the number of unsatisfied bonds over two.
+// Every thread of the block calls it.
 template <typename RowT, int LAYOUT, class RowSource>
 __device__ __forceinline__ void write_lattice(int32_t L, int64_t W, int64_t w, const RowSource &rows, void *lattice,
                                               int32_t *energy)
 {
+    __shared__ RowT first[kMaxStrips][32];   // first row of each strip
+    __shared__ int32_t bonds[kMaxStrips][32];
+    const int lane = threadIdx.x & 31, strip = threadIdx.x >> 5, strips = L / kStrip;
     const RowT mask = (L == (int)(8 * sizeof(RowT))) ? ~(RowT)0 : (((RowT)1 << L) - 1);
-    RowT first = 0, prev = 0;
+    RowT prev = 0;
     int unsat = 0;
-    for (int y = 0; y < L; ++y) {
-        const RowT r = rows(y);
-        const RowT rot = (r >> 1) | ((r & 1) << (L - 1));   // bit x = spin at x+1 (mod L)
-        unsat += __popcll((unsigned long long)((r ^ rot) & mask));
-        if (y == 0)
-            first = r;
-        else
-            unsat += __popcll((unsigned long long)((r ^ prev) & mask));
-        prev = r;
-        if (LAYOUT == MUCA_LAYOUT_PACKED) {
-            reinterpret_cast<RowT *>(lattice)[(size_t)y * W + w] = r;
-        } else {
-            int8_t *g = reinterpret_cast<int8_t *>(lattice);
-            for (int x = 0; x < L; ++x)
-                g[(size_t)(y * L + x) * W + w] = bit_at(r, x) ? (int8_t)-1 : (int8_t)1;
+    if (w < W) {
+        for (int i = 0; i < kStrip; ++i) {
+            const int y = strip * kStrip + i;
+            const RowT r = rows(y);
+            const RowT rot = (r >> 1) | ((r & 1) << (L - 1));   // bit x = spin at x+1 (mod L)
+            unsat += __popcll((unsigned long long)((r ^ rot) & mask));
+            if (i == 0)
+                first[strip][lane] = r;
+            else
+                unsat += __popcll((unsigned long long)((r ^ prev) & mask));
+            prev = r;
+            if (LAYOUT == MUCA_LAYOUT_PACKED) {
+                reinterpret_cast<RowT *>(lattice)[(size_t)y * W + w] = r;
+            } else {
+                int8_t *g = reinterpret_cast<int8_t *>(lattice);
+                for (int x = 0; x < L; ++x)
+                    g[(size_t)(y * L + x) * W + w] = bit_at(r, x) ? (int8_t)-1 : (int8_t)1;
+            }
         }
     }
-    unsat += __popcll((unsigned long long)((prev ^ first) & mask));   // row L-1 to row 0
-    energy[w] = unsat / 2;
+    __syncthreads();
+    if (w < W) {   // the strip's last row to the next strip's first (row L-1 to row 0)
+        const RowT next = first[strip + 1 < strips ? strip + 1 : 0][lane];
+        bonds[strip][lane] = unsat + __popcll((unsigned long long)((prev ^ next) & mask));
+    }
+    __syncthreads();
+    if (w < W && strip == 0) {
+        unsat = 0;
+        for (int i = 0; i < strips; ++i)
+            unsat += bonds[i][lane];
+        energy[w] = unsat / 2;
+    }
 }
 
 template <typename RowT>
@@ -67,52 +91,78 @@ template <typename RowT>
 struct GivenRows {
     int32_t L;
     const int8_t *spins;   // this walker's N spins, +1 / -1
+    bool words;            // whether they can be read as 4-byte words
     __device__ RowT operator()(int y) const
     {
         RowT r = 0;
-        for (int x = 0; x < L; ++x)
-            r |= (RowT)(spins[y * L + x] < 0) << x;
+        for (int x = 0; x < L; x += 4) {
+            const int8_t *p = spins + y * L + x;
+            if (words)
+                r |= (RowT)gather_signs(*reinterpret_cast<const uint32_t *>(p)) << x;
+            else
+                for (int u = 0; u < 4; ++u)
+                    r |= (RowT)(p[u] < 0) << (x + u);
+        }
         return r;
     }
 };
 
 template <typename RowT, int LAYOUT>
-__global__ void init_kernel(int32_t L, int64_t W, uint64_t seed, uint32_t walker0, void *lattice, int32_t *energy)
+__global__ void __launch_bounds__(32 * kMaxStrips) init_kernel(int32_t L, int64_t W, uint64_t seed, uint32_t walker0,
+                                                               void *lattice, int32_t *energy)
 {
-    const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (w >= W)
-        return;
+    const int64_t w = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
     const InitRows<RowT> rows{L, (uint32_t)seed, (uint32_t)(seed >> 32), walker0 + (uint32_t)w};
     write_lattice<RowT, LAYOUT>(L, W, w, rows, lattice, energy);
 }
 
 // Lattices given as int8 in[walker][site] (+1 / -1) into the layout, energies recomputed.
 template <typename RowT, int LAYOUT>
-__global__ void pack_kernel(int32_t L, int64_t W, const int8_t *in, void *lattice, int32_t *energy)
+__global__ void __launch_bounds__(32 * kMaxStrips) pack_kernel(int32_t L, int64_t W, const int8_t *in, void *lattice,
+                                                               int32_t *energy)
 {
-    const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (w >= W)
-        return;
-    const GivenRows<RowT> rows{L, in + (size_t)w * (size_t)(L * L)};
+    const int64_t w = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
+    const GivenRows<RowT> rows{L, in + (size_t)w * (size_t)(L * L), reinterpret_cast<uintptr_t>(in) % 4 == 0};
     write_lattice<RowT, LAYOUT>(L, W, w, rows, lattice, energy);
 }
 
+// The layout to int8 out[walker][site]: bound by memory, a transposition for int8.  A thread
+// writes 16 consecutive sites of its walker (L is a multiple of four, N of 16), which it
+// reads coalesced over the lanes, all at once.  One thread per walker and a byte at a time
+// took 539 us for L = 32 and 16384 walkers of bytes (16.8 MB each way), this 13 (2.6 TB/s).
+constexpr int kUnpackWarps = 8;
+
 template <typename RowT, int LAYOUT>
-__global__ void unpack_kernel(int32_t L, int64_t W, const void *lattice, int8_t *out)
+__global__ void __launch_bounds__(32 * kUnpackWarps) unpack_kernel(int32_t L, int64_t W, const void *lattice, int8_t *out)
 {
-    const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (w >= W)
+    const int64_t w = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
+    const int N = L * L, i0 = 16 * (int)(blockIdx.y * kUnpackWarps + (threadIdx.x >> 5));
+    if (w >= W || i0 >= N)
         return;
-    const int N = L * L;
-    for (int i = 0; i < N; ++i) {
-        int8_t v;
-        if (LAYOUT == MUCA_LAYOUT_PACKED) {
-            const RowT r = reinterpret_cast<const RowT *>(lattice)[(size_t)(i / L) * W + w];
-            v = bit_at(r, i % L) ? (int8_t)-1 : (int8_t)1;
-        } else {
-            v = reinterpret_cast<const int8_t *>(lattice)[(size_t)i * W + w];
+    uint32_t v[4];
+    if (LAYOUT == MUCA_LAYOUT_PACKED) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {   // four sites lie in one row
+            const int y = (i0 + 4 * j) / L, x = i0 + 4 * j - y * L;
+            v[j] = spread_signs((uint32_t)(reinterpret_cast<const RowT *>(lattice)[(size_t)y * W + w] >> x) & 15u);
         }
-        out[(size_t)w * N + i] = v;
+    } else {
+        const uint8_t *g = reinterpret_cast<const uint8_t *>(lattice) + (size_t)i0 * W + w;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            v[j] = 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                v[j] |= (uint32_t)g[(size_t)(4 * j + u) * W] << (8 * u);
+        }
+    }
+    int8_t *o = out + (size_t)w * N + i0;
+    if (reinterpret_cast<uintptr_t>(out) % 16 == 0) {
+        *reinterpret_cast<uint4 *>(o) = make_uint4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+            o[j] = (int8_t)(v[j / 4] >> (8 * (j % 4)));
     }
 }
 
@@ -239,8 +289,8 @@ cudaError_t launch_init(int32_t L, int32_t layout, int64_t W, uint64_t seed, uin
                         int32_t *energy,
                         cudaStream_t s)
 {
-    const int threads = 128;
-    const unsigned blocks = (unsigned)((W + threads - 1) / threads);
+    const int threads = 32 * (L / kStrip);
+    const unsigned blocks = (unsigned)((W + 31) / 32);
     if (L <= 32) {
         if (layout == MUCA_LAYOUT_PACKED)
             init_kernel<uint32_t, MUCA_LAYOUT_PACKED><<<blocks, threads, 0, s>>>(L, W, seed, walker0, lattice, energy);
@@ -258,8 +308,8 @@ cudaError_t launch_init(int32_t L, int32_t layout, int64_t W, uint64_t seed, uin
 cudaError_t launch_pack(int32_t L, int32_t layout, int64_t W, const int8_t *in, void *lattice, int32_t *energy,
                         cudaStream_t s)
 {
-    const int threads = 128;
-    const unsigned blocks = (unsigned)((W + threads - 1) / threads);
+    const int threads = 32 * (L / kStrip);
+    const unsigned blocks = (unsigned)((W + 31) / 32);
     if (L <= 32) {
         if (layout == MUCA_LAYOUT_PACKED)
             pack_kernel<uint32_t, MUCA_LAYOUT_PACKED><<<blocks, threads, 0, s>>>(L, W, in, lattice, energy);
@@ -276,8 +326,8 @@ cudaError_t launch_pack(int32_t L, int32_t layout, int64_t W, const int8_t *in, 
 
 cudaError_t launch_unpack(int32_t L, int32_t layout, int64_t W, const void *lattice, int8_t *out, cudaStream_t s)
 {
-    const int threads = 128;
-    const unsigned blocks = (unsigned)((W + threads - 1) / threads);
+    const int threads = 32 * kUnpackWarps;
+    const dim3 blocks((unsigned)((W + 31) / 32), (unsigned)((L * L + 16 * kUnpackWarps - 1) / (16 * kUnpackWarps)));
     if (L <= 32) {
         if (layout == MUCA_LAYOUT_PACKED)
             unpack_kernel<uint32_t, MUCA_LAYOUT_PACKED><<<blocks, threads, 0, s>>>(L, W, lattice, out);

@@ -147,3 +147,35 @@ def test_batch_across_counter_word(M):
                 m.close()
         for x, y in zip(alone, together):
             assert all(np.array_equal(p, q) for p, q in zip(x, y))
+
+
+@pytest.mark.parametrize("shift", [0, 4, 1])
+@pytest.mark.parametrize("L", [4, 8, 12, 20, 32, 36, 60, 64])
+def test_lattice_in_and_out(M, L, shift):
+    """Lattices given by the user come back unchanged, with their energies, from both
+    layouts, also where the allocator's buffer for them starts off a 16-byte boundary."""
+    import torch
+    from paper_1707_00919_gb300 import _lib as C
+    W, N = 71, L * L
+    held = {}
+
+    def alloc(n, ctx):
+        t = torch.empty(n + 16, dtype=torch.uint8, device="cuda")
+        p = t.data_ptr() + (shift if n == W * N else 0)   # the transfer buffer alone
+        held[p] = t
+        return p
+
+    spins = np.random.default_rng(L).choice(np.array([-1, 1], np.int8), size=(W, N))
+    s = spins.reshape(W, L, L).astype(np.int32)
+    bonds = (s != np.roll(s, 1, 1)).sum((1, 2)) + (s != np.roll(s, 1, 2)).sum((1, 2))
+    cb = C.ALLOC_FN(alloc), C.RELEASE_FN(lambda p, ctx: (held.pop(p), None)[1])
+    before = M._torch_cb or (C.ALLOC_FN(), C.RELEASE_FN())
+    assert C.load().muca_set_allocator(cb[0], cb[1], None) == 0
+    try:
+        for layout in (0, 1):
+            with M.Muca(L, W, 3, layout) as m:
+                m.set_lattice(spins)
+                assert np.array_equal(m.get_energies(), bonds // 2)
+                assert np.array_equal(np.asarray(m.get_lattice()).reshape(W, N), spins)
+    finally:
+        assert C.load().muca_set_allocator(before[0], before[1], None) == 0
