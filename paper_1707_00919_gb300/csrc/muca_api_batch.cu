@@ -1,6 +1,9 @@
 // muca_api_batch.cu - many instances in one launch of the batched persistent kernel
 // (one CUDA graph per weight iteration), the allocation-free batched sweep, and the
 // request server that admits simulations by device memory and advances them together.
+#include <functional>
+#include <queue>
+
 #include "muca_host.h"
 
 using namespace muca_host;
@@ -11,7 +14,7 @@ using namespace muca_host;
 struct muca_batch_s {
     std::vector<muca_t> inst;
     std::vector<cudaStream_t> saved_streams;
-    std::vector<int32_t> item_wpb;        // walkers per work item, per instance
+    std::vector<int32_t> item_wpb;        // most walkers per work item, per instance
     Allocator alloc;
     cudaStream_t stream = nullptr;
     void *block = nullptr;
@@ -35,27 +38,76 @@ namespace {
 
 bool batchable_L(int32_t L) { return L == 8 || L == 16 || L == 24 || L == 32 || L == 48 || L == 64; }
 
-// Work items of the given member instances (member index j refers to args[j]),
-// largest first so that the dynamic schedule ends evenly.
+// Time of an item of `walkers` walkers in units of a warp's share of the sub-partition, per
+// sweep: a block has an SM to itself, so an attempt's time goes by the warps that share a
+// sub-partition (L = 64: 59 cycles alone, 93 for two), whether all their lanes hold walkers
+// or not.  The chain length of a member's iteration goes with N.
+int64_t item_time(int32_t N, int64_t walkers)
+{
+    const int64_t warps = (walkers + 31) / 32, share = (warps + 3) / 4;
+    return (int64_t)N * (25 + 34 * share);
+}
+
+// Work items of the given member instances (member index j refers to args[j]), longest
+// first so that the dynamic schedule ends evenly.  An item of all the walkers that fit a
+// block uses an SM best; one of kSmallItem walkers, a warp per sub-partition, ends earlier.
+// The members with the longest chains get small items as far as that shortens the
+// schedule, which is played through for each such choice.  (Twelve instances of L = 16 to
+// 64, three of them L = 64: on 70 SMs the long items ran 7.9 ms, the others done after 1.6;
+// with small items for L = 64 on 138 SMs the iteration takes 6.1.  Ordered by walkers times sites, an L = 64
+// item of few walkers also started last.)
+constexpr int32_t kSmallItem = 128;
+
 void build_items(muca_batch_t b, const std::vector<int32_t> &members)
 {
-    std::vector<std::pair<int64_t, muca::BatchItem>> v;
-    for (size_t j = 0; j < members.size(); ++j) {
-        const muca_t h = b->inst[(size_t)members[j]];
-        const int32_t wpb = b->item_wpb[(size_t)members[j]];
-        for (int64_t wb = 0; wb < h->W; wb += wpb) {
-            muca::BatchItem it;
-            it.inst = (int32_t)j;
-            it.wpb = wpb;
-            it.wbase = wb;
-            const int64_t cost = (int64_t)h->N * std::min<int64_t>(wpb, h->W - wb);
-            v.emplace_back(cost, it);
+    std::vector<std::pair<int64_t, muca::BatchItem>> v, best;
+    std::vector<int32_t> limits{INT32_MAX};   // members of at least this N: small items
+    size_t whole = 0;
+    for (int32_t j : members) {
+        const muca_t h = b->inst[(size_t)j];
+        whole += (size_t)((h->W + b->item_wpb[(size_t)j] - 1) / b->item_wpb[(size_t)j]);
+        limits.push_back(h->N);
+    }
+    std::sort(limits.begin(), limits.end(), std::greater<int32_t>());
+    limits.erase(std::unique(limits.begin(), limits.end()), limits.end());
+    if (whole > 16 * (size_t)b->grid)   // the last item of an SM is then a small part
+        limits.resize(1);
+    int64_t best_end = INT64_MAX;
+    for (int32_t limit : limits) {
+        v.clear();
+        for (size_t j = 0; j < members.size(); ++j) {
+            const muca_t h = b->inst[(size_t)members[j]];
+            const int32_t most = b->item_wpb[(size_t)members[j]];
+            const int32_t wpb = h->N >= limit ? std::min(most, kSmallItem) : most;
+            for (int64_t wb = 0; wb < h->W; wb += wpb) {
+                muca::BatchItem it;
+                it.inst = (int32_t)j;
+                it.wpb = wpb;
+                it.wbase = wb;
+                v.emplace_back(item_time(h->N, std::min<int64_t>(wpb, h->W - wb)), it);
+            }
+        }
+        std::stable_sort(v.begin(), v.end(), [](const auto &x, const auto &y) { return x.first > y.first; });
+        int64_t end = 0;
+        if (limits.size() > 1) {
+            std::priority_queue<int64_t, std::vector<int64_t>, std::greater<int64_t>> free_at;
+            for (int i = 0; i < b->grid; ++i)
+                free_at.push(0);
+            for (const auto &x : v) {
+                const int64_t t = free_at.top() + x.first;
+                free_at.pop();
+                free_at.push(t);
+                end = std::max(end, t);
+            }
+        }
+        if (end < best_end) {
+            best_end = end;
+            best.swap(v);
         }
     }
-    std::stable_sort(v.begin(), v.end(), [](const auto &x, const auto &y) { return x.first > y.first; });
-    b->n_items = (int32_t)v.size();
-    for (size_t i = 0; i < v.size(); ++i)
-        b->h_items[i] = v[i].second;
+    b->n_items = (int32_t)best.size();
+    for (size_t i = 0; i < best.size(); ++i)
+        b->h_items[i] = best[i].second;
     b->members = members;
 }
 
@@ -419,7 +471,8 @@ int muca_batch_create(const muca_t *instances, int32_t n, muca_batch_t *out)
         b->item_wpb.push_back(wpb);
         b->smem = std::max(b->smem, muca::full_smem_bytes(h->L, wpb, true, false, stride));
         b->smem_launch = std::max(b->smem_launch, muca::launch_smem_bytes(h->L, wpb, false, stride));
-        items += (size_t)((h->W + wpb - 1) / wpb);
+        const int small = std::min(wpb, kSmallItem);
+        items += (size_t)((h->W + small - 1) / small);
     }
     b->items_capacity = items;
     cudaError_t err = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking);

@@ -179,3 +179,29 @@ def test_lattice_in_and_out(M, L, shift):
                 assert np.array_equal(np.asarray(m.get_lattice()).reshape(W, N), spins)
     finally:
         assert C.load().muca_set_allocator(before[0], before[1], None) == 0
+
+
+@pytest.mark.parametrize("specs", [
+    [(64, 300), (16, 700), (24, 129)],                  # small items for the longest chains
+    [(32, 128), (8, 31)],                               # one item each
+    [(8, 257)] * 5 + [(48, 383)],                       # ragged last items, alone and not
+    [(16, 40000), (64, 64)],                            # more items than SMs beside one long one
+])
+def test_batch_item_sizes(M, specs):
+    """Every choice of items covers every walker once: a batch equals its instances alone."""
+    out = []
+    for batched in (False, True):
+        inst = [M.Muca(L, W, 50 + i) for i, (L, W) in enumerate(specs)]
+        for m, (L, _) in zip(inst, specs):
+            m.set_weights(rand_weights(L, 3 * L))
+        if batched:
+            with M.Batch(inst) as b:
+                b.sweep(2, record=True)
+        else:
+            for m in inst:
+                m.sweep(2, record=True)
+        out.append([(m.get_histogram(), m.get_energies(), m.get_lattice()) for m in inst])
+        for m in inst:
+            m.close()
+    for x, y in zip(*out):
+        assert all(np.array_equal(p, q) for p, q in zip(x, y))
