@@ -20,7 +20,7 @@ struct muca_batch_s {
     void *block = nullptr;
     muca::SweepArgs *d_args = nullptr;    // [2 n]: thermalization, recording (with n_therm: both)
     muca::BatchItem *d_items = nullptr;   // capacity: all items of all instances
-    uint32_t *d_counter = nullptr;        // two work counters
+    uint32_t *d_work = nullptr;           // work counters, and a word per item
     muca::SweepArgs *h_args = nullptr;    // pinned staging of d_args
     muca::BatchItem *h_items = nullptr;   // pinned staging of d_items
     cudaEvent_t staged = nullptr;         // the last upload of h_args / h_items has completed
@@ -177,15 +177,13 @@ int build_graph(muca_batch_t b)
     if (err == cudaSuccess)
         err = cudaMemcpyAsync(b->d_args, b->h_args, sizeof(muca::SweepArgs) * 2 * nm, cudaMemcpyHostToDevice,
                               b->stream);
-    if (err == cudaSuccess)
-        err = cudaMemsetAsync(b->d_counter, 0, 2 * sizeof(uint32_t), b->stream);
     for (int32_t j : b->members) {
         const muca_t h = b->inst[(size_t)j];
         if (err == cudaSuccess)
             err = cudaMemsetAsync(h->d_hist, 0, sizeof(unsigned long long) * ((size_t)h->N + 1), b->stream);
     }
     if (err == cudaSuccess)
-        err = muca::launch_batch(b->d_args + nm, b->d_items, b->n_items, b->d_counter + 1, b->grid, b->smem_launch, true,
+        err = muca::launch_batch(b->d_args + nm, b->d_items, b->n_items, b->d_work, b->grid, b->smem_launch, true,
                                  b->stream);
     for (int32_t j : b->members) {
         const muca_t h = b->inst[(size_t)j];
@@ -313,8 +311,7 @@ int batch_run_iteration(muca_batch_t b, const std::vector<int32_t> &active, cons
         MUCA_CUDA(cudaMemcpyAsync(b->d_args, b->h_args, sizeof(muca::SweepArgs) * 2 * nm, cudaMemcpyHostToDevice,
                                   b->stream),
                   "batch descriptor upload");
-        MUCA_CUDA(cudaMemsetAsync(b->d_counter, 0, 2 * sizeof(uint32_t), b->stream), "work counter reset");
-        MUCA_CUDA(muca::launch_batch(b->d_args, b->d_items, b->n_items, b->d_counter, b->grid, b->smem_launch, false,
+        MUCA_CUDA(muca::launch_batch(b->d_args, b->d_items, b->n_items, b->d_work, b->grid, b->smem_launch, false,
                                      b->stream),
                   "batched thermalization");
         for (int32_t j : active) {
@@ -323,7 +320,7 @@ int batch_run_iteration(muca_batch_t b, const std::vector<int32_t> &active, cons
                       "histogram reset");
         }
         for (uint64_t done = 0;;) {
-            MUCA_CUDA(muca::launch_batch(b->d_args + nm, b->d_items, b->n_items, b->d_counter + 1, b->grid, b->smem_launch,
+            MUCA_CUDA(muca::launch_batch(b->d_args + nm, b->d_items, b->n_items, b->d_work, b->grid, b->smem_launch,
                                          true, b->stream),
                       "batched recording");
             done += cap;
@@ -342,7 +339,6 @@ int batch_run_iteration(muca_batch_t b, const std::vector<int32_t> &active, cons
             MUCA_CUDA(cudaMemcpyAsync(b->d_args + nm, b->h_args + nm, sizeof(muca::SweepArgs) * nm,
                                       cudaMemcpyHostToDevice, b->stream),
                       "batch descriptor upload");
-            MUCA_CUDA(cudaMemsetAsync(b->d_counter + 1, 0, sizeof(uint32_t), b->stream), "work counter reset");
         }
         rc = read_back(b, active);
         if (rc)
@@ -493,13 +489,13 @@ int muca_batch_create(const muca_t *instances, int32_t n, muca_batch_t *out)
         return cleanup(fail(MUCA_EINVAL, "batched kernel does not fit an SM with %zu bytes of shared memory", b->smem));
     b->grid = sms * occ;
     const size_t off_items = align256(sizeof(muca::SweepArgs) * 2 * (size_t)n);
-    const size_t off_counter = off_items + align256(sizeof(muca::BatchItem) * items);
-    b->block = device_alloc(b->alloc, off_counter + 256);
+    const size_t off_work = off_items + align256(sizeof(muca::BatchItem) * items);
+    b->block = device_alloc(b->alloc, off_work + align256(sizeof(uint32_t) * (2 + items)));
     if (!b->block)
         return cleanup(fail(MUCA_ENOMEM, "batch device allocation failed"));
     b->d_args = static_cast<muca::SweepArgs *>(b->block);
     b->d_items = reinterpret_cast<muca::BatchItem *>(static_cast<char *>(b->block) + off_items);
-    b->d_counter = reinterpret_cast<uint32_t *>(static_cast<char *>(b->block) + off_counter);
+    b->d_work = reinterpret_cast<uint32_t *>(static_cast<char *>(b->block) + off_work);
     err = cudaMallocHost(reinterpret_cast<void **>(&b->h_args), sizeof(muca::SweepArgs) * 2 * (size_t)n);
     if (err == cudaSuccess)
         err = cudaMallocHost(reinterpret_cast<void **>(&b->h_items), sizeof(muca::BatchItem) * items);
@@ -593,8 +589,7 @@ int muca_batch_sweep(muca_batch_t b, uint64_t n_sweeps, int record)
                                   cudaMemcpyHostToDevice, b->stream),
                   "batch descriptor upload");
         MUCA_CUDA(cudaEventRecord(b->staged, b->stream), "batch upload event");
-        MUCA_CUDA(cudaMemsetAsync(b->d_counter, 0, sizeof(uint32_t), b->stream), "work counter reset");
-        MUCA_CUDA(muca::launch_batch(b->d_args, b->d_items, b->n_items, b->d_counter, b->grid, b->smem_launch, record != 0,
+        MUCA_CUDA(muca::launch_batch(b->d_args, b->d_items, b->n_items, b->d_work, b->grid, b->smem_launch, record != 0,
                                      b->stream),
                   "batched launch");
         n_sweeps -= chunk;

@@ -220,11 +220,11 @@ cudaError_t launch_full_L64(const SweepArgs &a, int wpb, SweepForm form, bool re
 int resident_blocks(int L, int layout, int walkers_per_block);
 
 // Batched persistent kernel: allows `smem` bytes of dynamic shared memory, reports how
-// many blocks of it an SM holds, and launches it over a work list (counter zeroed by
-// the caller before every launch; L must be one of 8, 16, 24, 32, 48, 64).
+// many blocks of it an SM holds, and launches it over a work list (work: 2 + n_items words,
+// zeroed on the stream in front of it; L must be one of 8, 16, 24, 32, 48, 64).
 cudaError_t configure_batch(size_t smem);
 int batch_resident_blocks(size_t smem);
-cudaError_t launch_batch(const SweepArgs *insts, const BatchItem *items, int32_t n_items, uint32_t *counter,
+cudaError_t launch_batch(const SweepArgs *insts, const BatchItem *items, int32_t n_items, uint32_t *work,
                          int grid, size_t smem, bool record, cudaStream_t s);
 // Allocation-free batched sweep (see muca_batch_sweep_noalloc in muca.h): descriptors,
 // walkers per item and the prefix sums of the work items per instance (prefix[0] = 0,
