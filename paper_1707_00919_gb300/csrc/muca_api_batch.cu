@@ -23,7 +23,10 @@ struct muca_batch_s {
     uint32_t *d_work = nullptr;           // work counters, and a word per item
     muca::SweepArgs *h_args = nullptr;    // pinned staging of d_args
     muca::BatchItem *h_items = nullptr;   // pinned staging of d_items
-    cudaEvent_t staged = nullptr;         // the last upload of h_args / h_items has completed
+    muca::BatchJob *d_jobs = nullptr;     // [n]: weights in and histograms out, by member
+    muca::BatchJob *h_jobs = nullptr;     // pinned staging of d_jobs
+    int32_t bins = 0;                     // most bins of a member
+    cudaEvent_t staged = nullptr;         // the last upload of h_args / h_items / h_jobs has completed
     size_t items_capacity = 0;
     int32_t n_items = 0;                  // items of the current member set
     std::vector<int32_t> members;         // instances in the current work list
@@ -105,6 +108,12 @@ void build_items(muca_batch_t b, const std::vector<int32_t> &members)
             best.swap(v);
         }
     }
+    b->bins = 0;
+    for (size_t j = 0; j < members.size(); ++j) {
+        const muca_t h = b->inst[(size_t)members[j]];
+        b->h_jobs[j] = {{h->h_lnW, h->d_lnW, h->d_table, h->d_hist, h->N}, h->d_err, h->h_err, h->h_hist};
+        b->bins = std::max(b->bins, h->N + 1);
+    }
     b->n_items = (int32_t)best.size();
     for (size_t i = 0; i < best.size(); ++i)
         b->h_items[i] = best[i].second;
@@ -140,6 +149,9 @@ int upload_items(muca_batch_t b)
     MUCA_CUDA(cudaMemcpyAsync(b->d_items, b->h_items, sizeof(muca::BatchItem) * (size_t)b->n_items,
                               cudaMemcpyHostToDevice, b->stream),
               "batch work list upload");
+    MUCA_CUDA(cudaMemcpyAsync(b->d_jobs, b->h_jobs, sizeof(muca::BatchJob) * b->members.size(), cudaMemcpyHostToDevice,
+                              b->stream),
+              "batch member list upload");
     MUCA_CUDA(cudaEventRecord(b->staged, b->stream), "batch upload event");
     return MUCA_OK;
 }
@@ -154,10 +166,11 @@ int check_members(muca_batch_t b)
     return MUCA_OK;
 }
 
-// Captures one weight iteration of the current members: table uploads, the launch
-// descriptors, zeroed histograms, one launch that runs every member's thermalization and
-// then its recorded attempts (the recording descriptors carry n_therm), histogram and
-// error-word reads.  The host refills the pinned buffers before every replay.
+// Captures one weight iteration of the current members: the launch descriptors, one kernel
+// that builds every table and zeroes every histogram, one that runs every member's
+// thermalization and then its recorded attempts (the recording descriptors carry n_therm),
+// one that reads histograms and error words back.  The host refills the pinned buffers
+// before every replay.
 int build_graph(muca_batch_t b)
 {
     if (b->exec) {
@@ -167,32 +180,15 @@ int build_graph(muca_batch_t b)
     const size_t nm = b->members.size();
     cudaGraph_t g = nullptr;
     MUCA_CUDA(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal), "graph capture begin");
-    cudaError_t err = cudaSuccess;
-    for (int32_t j : b->members) {
-        const muca_t h = b->inst[(size_t)j];
-        if (err == cudaSuccess)
-            err = cudaMemcpyAsync(h->d_table, h->h_table, sizeof(uint32_t) * 5 * ((size_t)h->N + 1),
-                                  cudaMemcpyHostToDevice, b->stream);
-    }
+    cudaError_t err = cudaMemcpyAsync(b->d_args, b->h_args, sizeof(muca::SweepArgs) * 2 * nm, cudaMemcpyHostToDevice,
+                                      b->stream);
     if (err == cudaSuccess)
-        err = cudaMemcpyAsync(b->d_args, b->h_args, sizeof(muca::SweepArgs) * 2 * nm, cudaMemcpyHostToDevice,
-                              b->stream);
-    for (int32_t j : b->members) {
-        const muca_t h = b->inst[(size_t)j];
-        if (err == cudaSuccess)
-            err = cudaMemsetAsync(h->d_hist, 0, sizeof(unsigned long long) * ((size_t)h->N + 1), b->stream);
-    }
+        err = muca::launch_batch_tables(b->d_jobs, (int32_t)nm, b->bins, b->stream);
     if (err == cudaSuccess)
         err = muca::launch_batch(b->d_args + nm, b->d_items, b->n_items, b->d_work, b->grid, b->smem_launch, true,
                                  b->stream);
-    for (int32_t j : b->members) {
-        const muca_t h = b->inst[(size_t)j];
-        if (err == cudaSuccess)
-            err = cudaMemcpyAsync(h->h_hist, h->d_hist, sizeof(unsigned long long) * ((size_t)h->N + 1),
-                                  cudaMemcpyDeviceToHost, b->stream);
-        if (err == cudaSuccess)
-            err = cudaMemcpyAsync(h->h_err, h->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, b->stream);
-    }
+    if (err == cudaSuccess)
+        err = muca::launch_batch_read(b->d_jobs, (int32_t)nm, b->bins, b->stream);
     cudaError_t end = cudaStreamEndCapture(b->stream, &g);
     if (err == cudaSuccess)
         err = end;
@@ -242,21 +238,6 @@ void iteration_counts(muca_t h, const muca_params &p, uint64_t &n_therm, uint64_
     }
 }
 
-// Reads the members' histograms and error words into their pinned buffers and waits.
-int read_back(muca_batch_t b, const std::vector<int32_t> &active)
-{
-    for (int32_t j : active) {
-        const muca_t h = b->inst[(size_t)j];
-        MUCA_CUDA(cudaMemcpyAsync(h->h_hist, h->d_hist, sizeof(unsigned long long) * ((size_t)h->N + 1),
-                                  cudaMemcpyDeviceToHost, b->stream),
-                  "histogram read");
-        MUCA_CUDA(cudaMemcpyAsync(h->h_err, h->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, b->stream),
-                  "error word read");
-    }
-    MUCA_CUDA(cudaStreamSynchronize(b->stream), "batch synchronize");
-    return MUCA_OK;
-}
-
 // One weight iteration of the members `active` (indices into b->inst): member j
 // thermalizes therm[j] attempts per walker and records rec[j], all members in one
 // replay of the iteration graph (one launch for both phases), or, when some member
@@ -289,7 +270,7 @@ int batch_run_iteration(muca_batch_t b, const std::vector<int32_t> &active, cons
         muca_t h = b->inst[(size_t)active[j]];
         // the member's own last upload (muca_set_weights) may still read its staging buffer
         MUCA_CUDA(cudaEventSynchronize(h->table_copied), "waiting for the member's weights upload");
-        build_table(h->L, h->lnW, h->h_table);
+        std::copy(h->lnW.begin(), h->lnW.end(), h->h_lnW);
         b->h_args[j] = make_args(h, h->t, therm[j]);
         if (chunked) {   // a thermalization launch, then recording launches of at most cap attempts
             b->h_args[nm + j] = make_args(h, h->t + therm[j], std::min(rec[j], cap));
@@ -302,23 +283,13 @@ int batch_run_iteration(muca_batch_t b, const std::vector<int32_t> &active, cons
         MUCA_CUDA(cudaGraphLaunch(b->exec, b->stream), "batch iteration launch");
         MUCA_CUDA(cudaStreamSynchronize(b->stream), "batch synchronize");
     } else {
-        for (int32_t j : active) {
-            const muca_t h = b->inst[(size_t)j];
-            MUCA_CUDA(cudaMemcpyAsync(h->d_table, h->h_table, sizeof(uint32_t) * 5 * ((size_t)h->N + 1),
-                                      cudaMemcpyHostToDevice, b->stream),
-                      "table upload");
-        }
         MUCA_CUDA(cudaMemcpyAsync(b->d_args, b->h_args, sizeof(muca::SweepArgs) * 2 * nm, cudaMemcpyHostToDevice,
                                   b->stream),
                   "batch descriptor upload");
+        MUCA_CUDA(muca::launch_batch_tables(b->d_jobs, (int32_t)nm, b->bins, b->stream), "batch tables");
         MUCA_CUDA(muca::launch_batch(b->d_args, b->d_items, b->n_items, b->d_work, b->grid, b->smem_launch, false,
                                      b->stream),
                   "batched thermalization");
-        for (int32_t j : active) {
-            const muca_t h = b->inst[(size_t)j];
-            MUCA_CUDA(cudaMemsetAsync(h->d_hist, 0, sizeof(unsigned long long) * ((size_t)h->N + 1), b->stream),
-                      "histogram reset");
-        }
         for (uint64_t done = 0;;) {
             MUCA_CUDA(muca::launch_batch(b->d_args + nm, b->d_items, b->n_items, b->d_work, b->grid, b->smem_launch,
                                          true, b->stream),
@@ -340,9 +311,8 @@ int batch_run_iteration(muca_batch_t b, const std::vector<int32_t> &active, cons
                                       cudaMemcpyHostToDevice, b->stream),
                       "batch descriptor upload");
         }
-        rc = read_back(b, active);
-        if (rc)
-            return rc;
+        MUCA_CUDA(muca::launch_batch_read(b->d_jobs, (int32_t)nm, b->bins, b->stream), "batch read-back");
+        MUCA_CUDA(cudaStreamSynchronize(b->stream), "batch synchronize");
     }
     for (size_t j = 0; j < nm; ++j)
         b->inst[(size_t)active[j]]->t += therm[j] + rec[j];
@@ -490,15 +460,19 @@ int muca_batch_create(const muca_t *instances, int32_t n, muca_batch_t *out)
     b->grid = sms * occ;
     const size_t off_items = align256(sizeof(muca::SweepArgs) * 2 * (size_t)n);
     const size_t off_work = off_items + align256(sizeof(muca::BatchItem) * items);
-    b->block = device_alloc(b->alloc, off_work + align256(sizeof(uint32_t) * (2 + items)));
+    const size_t off_jobs = off_work + align256(sizeof(uint32_t) * (2 + items));
+    b->block = device_alloc(b->alloc, off_jobs + sizeof(muca::BatchJob) * (size_t)n);
     if (!b->block)
         return cleanup(fail(MUCA_ENOMEM, "batch device allocation failed"));
     b->d_args = static_cast<muca::SweepArgs *>(b->block);
     b->d_items = reinterpret_cast<muca::BatchItem *>(static_cast<char *>(b->block) + off_items);
     b->d_work = reinterpret_cast<uint32_t *>(static_cast<char *>(b->block) + off_work);
+    b->d_jobs = reinterpret_cast<muca::BatchJob *>(static_cast<char *>(b->block) + off_jobs);
     err = cudaMallocHost(reinterpret_cast<void **>(&b->h_args), sizeof(muca::SweepArgs) * 2 * (size_t)n);
     if (err == cudaSuccess)
         err = cudaMallocHost(reinterpret_cast<void **>(&b->h_items), sizeof(muca::BatchItem) * items);
+    if (err == cudaSuccess)
+        err = cudaMallocHost(reinterpret_cast<void **>(&b->h_jobs), sizeof(muca::BatchJob) * (size_t)n);
     if (err != cudaSuccess)
         return cleanup(cuda_fail(err, "batch pinned buffers"));
     // from now on every call on a member instance is ordered with the batch's work
@@ -528,6 +502,8 @@ int muca_batch_destroy(muca_batch_t b)
         cudaFreeHost(b->h_args);
     if (b->h_items)
         cudaFreeHost(b->h_items);
+    if (b->h_jobs)
+        cudaFreeHost(b->h_jobs);
     if (b->staged)
         cudaEventDestroy(b->staged);
     if (b->stream)

@@ -154,10 +154,7 @@ int muca_iterate_until_flat(muca_t h, const muca_params *p_in, muca_stats *stats
                 full = prev_width == N + 1;
             }
         }
-        rc = upload_table(h);
-        if (rc)
-            return rc;
-        rc = muca_reset_histogram(h);
+        rc = upload_table(h, true);
         if (rc)
             return rc;
         rc = run_therm_record(h, n_therm, n_upd);

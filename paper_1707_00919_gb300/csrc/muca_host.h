@@ -41,6 +41,11 @@ void device_free(const Allocator &a, void *p);
 
 constexpr size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
+// The error word's place in front of the histogram, so that both come with one copy.
+constexpr size_t kErrBytes = 256;
+// Energies up to this size are read through pinned memory together with the error word.
+constexpr size_t kEnergyStageBytes = 256 * 1024;
+
 // Largest attempts per walker one recorded launch may take so that a block's 32-bit
 // shared histogram bins cannot overflow (each walker adds one count per attempt).
 inline uint64_t max_recorded_attempts(int wpb) { return 0xFFFFFFFFull / (uint64_t)std::max(wpb, 256); }
@@ -72,10 +77,12 @@ struct muca_s {
     uint32_t *d_table = nullptr;
     unsigned long long *d_hist = nullptr;
     uint32_t *d_err = nullptr;
-    uint32_t *h_table = nullptr;     // pinned staging of the table upload
-    unsigned long long *h_hist = nullptr;  // pinned staging of histogram reads
-    uint32_t *h_err = nullptr;
-    cudaEvent_t table_copied = nullptr;    // last table upload has left h_table
+    void *pinned = nullptr;          // single pinned allocation holding the host buffers
+    double *h_lnW = nullptr;         // weights as the table kernel reads them
+    int32_t *h_energy = nullptr;     // staging of energy reads, followed by h_err; null for many walkers
+    uint32_t *h_err = nullptr;       // kErrBytes, followed by h_hist, as on the device
+    unsigned long long *h_hist = nullptr;  // staging of histogram reads
+    cudaEvent_t table_copied = nullptr;    // the last table kernel has read h_lnW
     std::vector<double> lnW;
     void *iter_block = nullptr;      // device iteration state (muca_iterate_device)
     double *d_lnW = nullptr;         // device ln W (in block): the table is built from it
@@ -98,7 +105,8 @@ namespace muca_host {
 // Instance helpers (muca_api.cu).
 // Acceptance thresholds from ln W (Sec. 2.3, integer form): see muca.h.
 void build_table(int32_t L, const std::vector<double> &lnW, uint32_t *T);
-int upload_table(muca_t h);
+// The weights to the device and the table built from them; zero_hist: the histogram zeroed too.
+int upload_table(muca_t h, bool zero_hist = false);
 int check_device_error(muca_t h);
 int sync_and_check(muca_t h);
 // Which instances have sweeps that the host has not waited for, so that a launch knows

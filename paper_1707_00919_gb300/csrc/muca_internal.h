@@ -148,9 +148,26 @@ cudaError_t launch_iter_recursion(const IterState *st, int32_t N, double *lnW, c
                                   cudaStream_t s);
 cudaError_t launch_iter_table(const IterState *st, int32_t N, const double *lnW, uint32_t *table, cudaStream_t s);
 
-// Thresholds T[e][k] of the weights lnW[N + 1] on the device (the host's build_table
-// arithmetic, bit for bit): every weight upload of an instance.
-cudaError_t launch_table(int32_t N, const double *lnW, uint32_t *table, cudaStream_t s);
+// New weights of an instance: src[N + 1] (pinned host memory) to lnW, thresholds T[e][k]
+// (the host's build_table arithmetic, bit for bit), the histogram zeroed unless hist is null.
+struct TableJob {
+    const double *src;
+    double *lnW;
+    uint32_t *table;
+    unsigned long long *hist;
+    int32_t N;
+};
+cudaError_t launch_table(const TableJob &job, cudaStream_t s);
+
+// The same for all members of a batch (jobs in device memory, bins: the most of any).
+struct BatchJob {
+    TableJob table;
+    const uint32_t *err;            // to h_err and, with the histogram, h_hist (pinned)
+    uint32_t *h_err;
+    unsigned long long *h_hist;
+};
+cudaError_t launch_batch_tables(const BatchJob *jobs, int32_t n, int32_t bins, cudaStream_t s);
+cudaError_t launch_batch_read(const BatchJob *jobs, int32_t n, int32_t bins, cudaStream_t s);
 
 // One work item of the batched kernel: walkers wbase .. wbase + wpb - 1 of instance inst.
 struct BatchItem {

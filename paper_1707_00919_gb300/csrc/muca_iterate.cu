@@ -3,6 +3,7 @@
 // and the threshold table of the next iteration.  Every floating-point step is the one
 // the host library takes, in the same order (muca_math.cuh for exp and ln), so the
 // weights, tables and metrics are the host's bit for bit.
+#include <algorithm>
 #include <climits>
 #include <cstdint>
 
@@ -199,12 +200,45 @@ __global__ void iter_table_kernel(const IterState *st, int32_t N, const double *
         T[i] = table_entry(N, lnW, i);
 }
 
-// Thresholds of the given weights (every weight upload of an instance).
-__global__ void table_kernel(int32_t N, const double *lnW, uint32_t *T)
+// New weights of an instance, read where the host put them (see upload_table).
+__device__ __forceinline__ void run_table_job(const TableJob &job, int32_t i)
+{
+    if (i >= (job.N + 1) * 5)
+        return;
+    job.table[i] = table_entry(job.N, job.src, i);
+    if (i % 5 == 0) {
+        job.lnW[i / 5] = job.src[i / 5];
+        if (job.hist)
+            job.hist[i / 5] = 0ull;
+    }
+}
+
+__global__ void table_kernel(const TableJob job)
+{
+    run_table_job(job, blockIdx.x * blockDim.x + threadIdx.x);
+}
+
+// A batch's members, one row of blocks each.  One kernel before the sweeps and one after
+// them, where each member had two operations on either side and its table was built on the
+// host: 16 members of L = 16 with 1024 walkers, 668 us per
+// iteration of 41 sweeps, now 490.
+__global__ void batch_tables_kernel(const BatchJob *jobs, int32_t n)
+{
+    for (int32_t j = blockIdx.y; j < n; j += gridDim.y)
+        run_table_job(jobs[j].table, blockIdx.x * blockDim.x + threadIdx.x);
+}
+
+// Histograms and error words into the members' pinned buffers.
+__global__ void batch_read_kernel(const BatchJob *jobs, int32_t n)
 {
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < (N + 1) * 5)
-        T[i] = table_entry(N, lnW, i);
+    for (int32_t j = blockIdx.y; j < n; j += gridDim.y) {
+        const BatchJob &job = jobs[j];
+        if (i <= job.table.N)
+            job.h_hist[i] = job.table.hist[i];
+        if (i == 0)
+            *job.h_err = *job.err;
+    }
 }
 
 }  // namespace
@@ -238,10 +272,24 @@ cudaError_t launch_iter_recursion(const IterState *st, int32_t N, double *lnW, c
     return cudaGetLastError();
 }
 
-cudaError_t launch_table(int32_t N, const double *lnW, uint32_t *table, cudaStream_t s)
+cudaError_t launch_table(const TableJob &job, cudaStream_t s)
 {
-    const int32_t n = (N + 1) * 5;
-    table_kernel<<<(n + 127) / 128, 128, 0, s>>>(N, lnW, table);
+    const int32_t n = (job.N + 1) * 5;
+    table_kernel<<<(n + 127) / 128, 128, 0, s>>>(job);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_batch_tables(const BatchJob *jobs, int32_t n, int32_t bins, cudaStream_t s)
+{
+    const dim3 grid((unsigned)((bins * 5 + 127) / 128), (unsigned)std::min(n, 65535));
+    batch_tables_kernel<<<grid, 128, 0, s>>>(jobs, n);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_batch_read(const BatchJob *jobs, int32_t n, int32_t bins, cudaStream_t s)
+{
+    const dim3 grid((unsigned)((bins + 127) / 128), (unsigned)std::min(n, 65535));
+    batch_read_kernel<<<grid, 128, 0, s>>>(jobs, n);
     return cudaGetLastError();
 }
 
