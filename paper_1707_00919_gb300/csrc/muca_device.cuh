@@ -465,9 +465,9 @@ __device__ __forceinline__ uint32_t add_count(uint32_t w, int x, int m, uint32_t
 // 1 the row address if the next attempt flips, 2 also the address of its flipped candidate:
 // each step shortens the chain and adds instructions.  The histogram's reduction comes
 // after the loads, which it would delay.  Measured, us per sweep (EARLY 0 / 1 / 2):
-//   L = 32, 16 384 walkers, one warp per sub-partition      24.7 / 24.4 / 24.4
-//   L = 32, 38 912 walkers, two warps                       41.9 / 42.0 / 43.1
-//   L = 64, 32 768 walkers, 1.75 warps                      166  / 169  / 177
+//   L = 32, 16 384 walkers, one warp per sub-partition      24.7 / 24.4 / 24.5
+//   L = 32, 38 912 walkers, two warps                       41.9 / 41.8 / 43.4
+//   L = 64, 32 768 walkers, 1.75 warps                      166  / 168  / 176
 //   L = 32, 4096 walkers, chain warps with generators       18.7 / 18.2 / 17.7
 //   L = 64, 4096 walkers, the same                          74.8 / 74.2 / 72.1
 //   L = 8, 128 walkers, the same                            1.23 / 1.16 / 1.28
@@ -570,8 +570,8 @@ struct AttemptStream {
 // instructions instead of 27.2.  The decision enters as a factor 0 or 1: the step of the
 // energy row and the flip bit are multiply-adds, on the pipe with room, where a select
 // each would load the ALU.  Measured at L = 32, 48 640 walkers (2.5 warps per SM
-// sub-partition) 55.7 us per sweep against 62.8 with the look-ahead; L = 16, 77 824 walkers
-// (4 warps) 18.1 against 20.9; at one warp 33 against 24.9, at two 41 and 41 (L = 32, 38 912
+// sub-partition) 57.9 us per sweep against 61.5 with the look-ahead; L = 16, 77 824 walkers
+// (4 warps) 18.2 against 20.8; at one warp 33 against 24.5, at two 41 and 42 (L = 32, 38 912
 // walkers): launches of more than two warps per sub-partition take it.
 // ---------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t mad32(uint32_t a, uint32_t b, uint32_t c)

@@ -5,7 +5,11 @@
 // bound by its own instruction issue (one half-rate instruction per two cycles, a wide
 // multiply twice that): Philox is half of it.  Generator warps on the idle sub-partitions
 // draw the words into a ring in shared memory, a chunk of about 128 attempts at a time, and
-// the chain warp reads four words per 16-byte load.
+// the chain warp reads four words per 16-byte load.  What bounds it now is the chain warp's
+// issue again, 18 instructions per attempt.  Measured, us per sweep without and with the
+// generators: L = 8, 128 walkers 1.58 -> 1.19; L = 16, 4096 walkers 6.31 -> 4.41; L = 24,
+// 5003 walkers 14.2 -> 10.4; L = 32, 4096 walkers 24.5 -> 17.7; L = 48, 1024 walkers 56.6 ->
+// 42.2; L = 64, 9728 walkers 99.6 -> 73.4.
 #pragma once
 
 #include "muca_device.cuh"
