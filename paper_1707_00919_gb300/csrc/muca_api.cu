@@ -761,10 +761,8 @@ int muca_get_energies(muca_t h, int32_t *e_out, size_t n)
     MUCA_CUDA(cudaMemcpyAsync(h->h_energy, h->d_energy, bytes, cudaMemcpyDeviceToHost, h->stream),
               "energy and error word read");
     MUCA_CUDA(wait_stream(h), "stream synchronize");
-    rc = check_device_error(h);
-    if (rc == MUCA_OK)
-        std::copy(h->h_energy, h->h_energy + n, e_out);
-    return rc;
+    std::copy(h->h_energy, h->h_energy + n, e_out);
+    return check_device_error(h);
 }
 
 int muca_get_lattice(muca_t h, int8_t *out, size_t n)
