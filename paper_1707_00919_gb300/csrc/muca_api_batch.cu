@@ -30,6 +30,7 @@ struct muca_batch_s {
     size_t items_capacity = 0;
     int32_t n_items = 0;                  // items of the current member set
     std::vector<int32_t> members;         // instances in the current work list
+    uint64_t longest = 0;                 // longest chain that the work list was made for
     size_t smem = 0;                      // of the largest member's table and rows
     size_t smem_launch = 0;               // of a launch
     int grid = 0;
@@ -41,63 +42,64 @@ namespace {
 
 bool batchable_L(int32_t L) { return L == 8 || L == 16 || L == 24 || L == 32 || L == 48 || L == 64; }
 
-// Time of an item of `walkers` walkers in units of a warp's share of the sub-partition, per
-// sweep: a block has an SM to itself, so an attempt's time goes by the warps that share a
-// sub-partition (L = 64: 59 cycles alone, 93 for two), whether all their lanes hold walkers
-// or not.  The chain length of a member's iteration goes with N.
-int64_t item_time(int32_t N, int64_t walkers)
+// Time of an item of `walkers` walkers and `length` attempts each, in cycles: a block has an
+// SM to itself, so an attempt's time goes by the warps that share a sub-partition (L = 64:
+// 59 cycles alone, 93 for two), whether all their lanes hold walkers or not.
+double item_time(uint64_t length, int64_t walkers)
 {
     const int64_t warps = (walkers + 31) / 32, share = (warps + 3) / 4;
-    return (int64_t)N * (25 + 34 * share);
+    return (double)length * (double)(25 + 34 * share);
 }
 
 // Work items of the given member instances (member index j refers to args[j]), longest
 // first so that the dynamic schedule ends evenly.  An item of all the walkers that fit a
 // block uses an SM best; one of kSmallItem walkers, a warp per sub-partition, ends earlier.
-// The members with the longest chains get small items as far as that shortens the
-// schedule, which is played through for each such choice.  (Twelve instances of L = 16 to
-// 64, three of them L = 64: on 70 SMs the long items ran 7.9 ms, the others done after 1.6;
-// with small items for L = 64 on 138 SMs the iteration takes 6.1.  Ordered by walkers times sites, an L = 64
-// item of few walkers also started last.)
+// The members with the longest chains (lengths: attempts per walker of the iteration at
+// hand) get small items as far as that shortens the schedule, which is played through for
+// some such choices.  (Twelve instances of L = 16 to 64, three of them L = 64: on 70 SMs
+// the long items ran 7.9 ms, the others done after 1.6; with small items for L = 64 on 138
+// SMs the iteration takes 6.1.  With the Eq. (7) schedule the longest chains are those of
+// the fewest walkers: 24 requests served, L = 8 to 64, p50 3.1 s and 62 s in all when sizes
+// and order went by L, 1.8 s and 38 s now.)
 constexpr int32_t kSmallItem = 128;
 
-void build_items(muca_batch_t b, const std::vector<int32_t> &members)
+void build_items(muca_batch_t b, const std::vector<int32_t> &members, const std::vector<uint64_t> &lengths)
 {
-    std::vector<std::pair<int64_t, muca::BatchItem>> v, best;
-    std::vector<int32_t> limits{INT32_MAX};   // members of at least this N: small items
+    std::vector<std::pair<double, muca::BatchItem>> v, best;
+    std::vector<uint64_t> sorted(lengths), limits{UINT64_MAX};   // members of at least this length: small items
     size_t whole = 0;
     for (int32_t j : members) {
         const muca_t h = b->inst[(size_t)j];
         whole += (size_t)((h->W + b->item_wpb[(size_t)j] - 1) / b->item_wpb[(size_t)j]);
-        limits.push_back(h->N);
     }
-    std::sort(limits.begin(), limits.end(), std::greater<int32_t>());
-    limits.erase(std::unique(limits.begin(), limits.end()), limits.end());
-    if (whole > 16 * (size_t)b->grid)   // the last item of an SM is then a small part
-        limits.resize(1);
-    int64_t best_end = INT64_MAX;
-    for (int32_t limit : limits) {
+    std::sort(sorted.begin(), sorted.end(), std::greater<uint64_t>());
+    sorted.erase(std::unique(sorted.begin(), sorted.end()), sorted.end());
+    if (whole <= 16 * (size_t)b->grid)   // beyond that the last item of an SM is a small part
+        for (size_t i = 0; i < sorted.size(); i = i < 6 ? i + 1 : 2 * i)
+            limits.push_back(sorted[i]);
+    double best_end = INFINITY;
+    for (uint64_t limit : limits) {
         v.clear();
         for (size_t j = 0; j < members.size(); ++j) {
             const muca_t h = b->inst[(size_t)members[j]];
             const int32_t most = b->item_wpb[(size_t)members[j]];
-            const int32_t wpb = h->N >= limit ? std::min(most, kSmallItem) : most;
+            const int32_t wpb = lengths[j] >= limit ? std::min(most, kSmallItem) : most;
             for (int64_t wb = 0; wb < h->W; wb += wpb) {
                 muca::BatchItem it;
                 it.inst = (int32_t)j;
                 it.wpb = wpb;
                 it.wbase = wb;
-                v.emplace_back(item_time(h->N, std::min<int64_t>(wpb, h->W - wb)), it);
+                v.emplace_back(item_time(lengths[j], std::min<int64_t>(wpb, h->W - wb)), it);
             }
         }
         std::stable_sort(v.begin(), v.end(), [](const auto &x, const auto &y) { return x.first > y.first; });
-        int64_t end = 0;
+        double end = 0.0;
         if (limits.size() > 1) {
-            std::priority_queue<int64_t, std::vector<int64_t>, std::greater<int64_t>> free_at;
+            std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
             for (int i = 0; i < b->grid; ++i)
-                free_at.push(0);
+                free_at.push(0.0);
             for (const auto &x : v) {
-                const int64_t t = free_at.top() + x.first;
+                const double t = free_at.top() + x.first;
                 free_at.pop();
                 free_at.push(t);
                 end = std::max(end, t);
@@ -118,6 +120,7 @@ void build_items(muca_batch_t b, const std::vector<int32_t> &members)
     for (size_t i = 0; i < best.size(); ++i)
         b->h_items[i] = best[i].second;
     b->members = members;
+    b->longest = sorted.front();
 }
 
 muca::SweepArgs make_args(muca_t h, uint64_t t0, uint64_t n)
@@ -250,9 +253,14 @@ int batch_run_iteration(muca_batch_t b, const std::vector<int32_t> &active, cons
     int rc = stage_wait(b);
     if (rc)
         return rc;
-    if (active != b->members || !b->exec) {
+    std::vector<uint64_t> lengths(active.size());
+    for (size_t j = 0; j < active.size(); ++j)
+        lengths[j] = therm[j] + rec[j];
+    const uint64_t longest = *std::max_element(lengths.begin(), lengths.end());
+    // Eq. (7) makes chains grow and shrink: a new list when the longest has by a factor of two
+    if (active != b->members || !b->exec || longest / 2 > b->longest || longest < b->longest / 2) {
         MUCA_CUDA(cudaStreamSynchronize(b->stream), "batch synchronize");
-        build_items(b, active);
+        build_items(b, active, lengths);
         rc = upload_items(b);
         if (rc)
             return rc;
@@ -536,13 +544,16 @@ int muca_batch_sweep(muca_batch_t b, uint64_t n_sweeps, int record)
     for (muca_t h : b->inst)
         max_n = std::min<uint64_t>(max_n, (record ? 0xFFFFFFFFull / 256ull : UINT64_MAX) / (uint64_t)h->N);
     std::vector<int32_t> all(b->inst.size());
-    for (size_t i = 0; i < all.size(); ++i)
+    std::vector<uint64_t> lengths(b->inst.size());
+    for (size_t i = 0; i < all.size(); ++i) {
         all[i] = (int32_t)i;
+        lengths[i] = (uint64_t)b->inst[i]->N;
+    }
     int rc = stage_wait(b);
     if (rc)
         return rc;
     if (b->members != all) {
-        build_items(b, all);
+        build_items(b, all, lengths);
         if (b->exec) {
             cudaGraphExecDestroy(b->exec);
             b->exec = nullptr;
