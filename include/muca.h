@@ -232,7 +232,9 @@ int muca_get_site_order(muca_t h, int32_t *order);
 int muca_set_stream(muca_t h, void *cuda_stream);
 
 /* Replaces the device allocator used by later muca_create calls (alloc == NULL restores
- * cudaMalloc/cudaFree).  alloc(size, ctx) returns device memory or NULL. */
+ * cudaMalloc/cudaFree).  alloc(size, ctx) returns device memory or NULL, aligned to 8
+ * bytes (16 for MUCA_LAYOUT_INT8 instances whose walker count is a multiple of 16 and at
+ * least 32); calls given less return MUCA_EINVAL. */
 int muca_set_allocator(void *(*alloc)(size_t size, void *ctx), void (*release)(void *ptr, void *ctx),
                        void *ctx);
 
@@ -492,7 +494,9 @@ int muca_server_totals(muca_server_t s, uint64_t *walker_attempts, double *secon
  * lattice in `layout`, energy indices int32[n_walkers], thresholds uint32[(L*L+1)*5]
  * (as muca_get_table returns them), histogram uint64[L*L+1] (added to), error word
  * uint32 (bits OR-ed in, 0 = fine).  t0 is the attempt counter of the first attempt and
- * must lie on a sweep boundary (a multiple of L*L).  A walker whose energy index lies
+ * must lie on a sweep boundary (a multiple of L*L).  Every buffer is aligned to its element
+ * (4 or 8 bytes for packed rows), an int8 lattice whose n_walkers is a multiple of 16 and at
+ * least 32 to 16 bytes.  A walker whose energy index lies
  * outside 0..L*L sets bit 0 of the error word and is left unchanged; an index inside
  * that range that does not match the walker's lattice is used as given (flips whose
  * target energy leaves the grid are rejected: their thresholds are 0). */
@@ -523,7 +527,8 @@ typedef struct {
  * Errors: MUCA_EINVAL (NULL, more than MUCA_NOALLOC_MAX_INSTANCES instances, L outside
  * the list, t0 off a sweep boundary, a recorded launch longer than 0xFFFFFFFF / 256
  * attempts per walker, more than 2^31 - 1 work items of up to 256 walkers, two instances
- * whose lattice or energy buffers overlap, the same instance given twice included),
+ * whose lattice or energy buffers overlap, the same instance given twice included, a buffer
+ * off its alignment),
  * MUCA_ECUDA. */
 int muca_batch_sweep_noalloc(const muca_raw_instance *instances, int32_t n, uint64_t n_sweeps, int record,
                              void *cuda_stream);

@@ -535,6 +535,10 @@ int muca_create_ex(const muca_options *opt, muca_t *out)
     h->block = device_alloc(h->alloc, total);
     if (!h->block)
         return cleanup(fail(MUCA_ENOMEM, "device allocation of %zu bytes failed", total));
+    // the block begins with the lattice; weights and histogram are 64-bit
+    const size_t unit = std::max(lattice_alignment(L, h->layout, h->W), sizeof(uint64_t));
+    if (!aligned(h->block, unit))
+        return cleanup(fail(MUCA_EINVAL, "the allocator's memory is not aligned to %zu bytes", unit));
     char *base = static_cast<char *>(h->block);
     h->d_lattice = base + off_lat;
     h->d_energy = reinterpret_cast<int32_t *>(base + off_e);

@@ -472,6 +472,8 @@ int muca_batch_create(const muca_t *instances, int32_t n, muca_batch_t *out)
     b->block = device_alloc(b->alloc, off_jobs + sizeof(muca::BatchJob) * (size_t)n);
     if (!b->block)
         return cleanup(fail(MUCA_ENOMEM, "batch device allocation failed"));
+    if (!aligned(b->block, sizeof(uint64_t)))
+        return cleanup(fail(MUCA_EINVAL, "the allocator's memory is not aligned to %zu bytes", sizeof(uint64_t)));
     b->d_args = static_cast<muca::SweepArgs *>(b->block);
     b->d_items = reinterpret_cast<muca::BatchItem *>(static_cast<char *>(b->block) + off_items);
     b->d_work = reinterpret_cast<uint32_t *>(static_cast<char *>(b->block) + off_work);
@@ -690,6 +692,13 @@ int muca_batch_sweep_noalloc(const muca_raw_instance *instances, int32_t n, uint
             return fail(MUCA_EINVAL, "instance %d: n_walkers = %lld out of range", i, (long long)r.n_walkers);
         if (!r.lattice || !r.energy || !r.table || !r.hist || !r.err)
             return fail(MUCA_EINVAL, "instance %d: NULL device buffer", i);
+        // the kernel's accesses are as wide as these: off them, a fault instead of an error
+        const size_t lattice_unit = lattice_alignment(r.L, r.layout, r.n_walkers);
+        if (!aligned(r.lattice, lattice_unit))
+            return fail(MUCA_EINVAL, "instance %d: lattice not aligned to %zu bytes", i, lattice_unit);
+        if (!aligned(r.energy, sizeof(int32_t)) || !aligned(r.table, sizeof(uint32_t)) || !aligned(r.err, sizeof(uint32_t)) ||
+            (record && !aligned(r.hist, sizeof(unsigned long long))))
+            return fail(MUCA_EINVAL, "instance %d: energies, table, histogram or error word not aligned to their type", i);
         const uint64_t N = (uint64_t)r.L * (uint64_t)r.L;
         if (r.t0 % N != 0)
             return fail(MUCA_EINVAL, "instance %d: t0 is not at a sweep boundary", i);

@@ -302,6 +302,11 @@ int muca_iterate_device(muca_t h, const muca_params *p_in, int32_t iterations_pe
         h->iter_block = device_alloc(h->alloc, align256(sizeof(muca::IterState)));
         if (!h->iter_block)
             return fail(MUCA_ENOMEM, "device allocation for the iteration state failed");
+        if (!aligned(h->iter_block, alignof(muca::IterState))) {
+            device_free(h->alloc, h->iter_block);
+            h->iter_block = nullptr;
+            return fail(MUCA_EINVAL, "the allocator's memory is not aligned to %zu bytes", alignof(muca::IterState));
+        }
         h->d_iter = static_cast<muca::IterState *>(h->iter_block);
         MUCA_CUDA(cudaMallocHost(reinterpret_cast<void **>(&h->h_iter), sizeof(muca::IterState)),
                   "pinned iteration state");

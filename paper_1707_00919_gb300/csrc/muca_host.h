@@ -41,6 +41,16 @@ void device_free(const Allocator &a, void *p);
 
 constexpr size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
+// Alignment that the kernels need of a lattice: whole words of a packed row, and 16 bytes
+// where the bytes of 32 walkers are moved as vectors.
+inline size_t lattice_alignment(int32_t L, int32_t layout, int64_t W)
+{
+    if (layout == MUCA_LAYOUT_PACKED)
+        return L <= 32 ? sizeof(uint32_t) : sizeof(uint64_t);
+    return W >= 32 && W % 16 == 0 ? 16 : 1;
+}
+inline bool aligned(const void *p, size_t n) { return reinterpret_cast<uintptr_t>(p) % n == 0; }
+
 // The error word's place in front of the histogram, so that both come with one copy.
 constexpr size_t kErrBytes = 256;
 // Energies up to this size are read through pinned memory together with the error word.
