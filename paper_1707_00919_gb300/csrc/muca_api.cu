@@ -97,21 +97,27 @@ int check_device_error(muca_t h)
 
 namespace {
 
-std::mutex g_queued_mutex;
-std::vector<muca_t> g_queued;   // instances with sweeps that the host has not waited for
+std::mutex g_flights_mutex;
+std::vector<Flight *> g_flights;   // sweeps that the host has not seen the end of
 
-// Whether the instance's own stream has run dry.  A stream given by the caller is not
-// asked (the caller may have destroyed it): such an instance counts until it is waited for.
-// The query must not disturb a capture that another thread has under way.
-bool ran_dry(muca_t h)
-{
-    if (h->stream != h->own_stream)
-        return false;
+// Calls that ask or mark a stream must not disturb a capture that another thread has under way.
+struct RelaxedCapture {
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess)
+    bool set = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
+    ~RelaxedCapture()
+    {
+        if (set)
+            cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+};
+
+// Whether the sweeps have ended.
+bool landed(const Flight &f)
+{
+    const RelaxedCapture relaxed;
+    if (!relaxed.set)
         return false;
-    const cudaError_t err = cudaStreamQuery(h->stream);
-    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t err = f.ask ? cudaStreamQuery(f.ask) : cudaEventQuery(f.swept);
     if (err != cudaSuccess)
         cudaGetLastError();   // not ready is not an error of the launches to come
     return err == cudaSuccess;
@@ -119,48 +125,71 @@ bool ran_dry(muca_t h)
 
 }  // namespace
 
-bool sweeps_queued(muca_t h)
+bool device_alone(Flight &f)
 {
     constexpr int kRemembered = 8;   // launches for which an overlap is taken to recur
-    std::lock_guard<std::mutex> lock(g_queued_mutex);
-    bool alone = true;
-    if (h->company > 0) {   // no query (microseconds) while the overlaps go on
-        --h->company;
-        alone = false;
+    std::lock_guard<std::mutex> lock(g_flights_mutex);
+    if (f.company > 0) {   // no query (microseconds) while the overlaps go on
+        --f.company;
+        return false;
     }
-    bool listed = false;
-    for (size_t i = 0; i < g_queued.size(); ++i) {
-        const muca_t o = g_queued[i];
-        if (o == h) {
-            listed = true;
-        } else if (o->device == h->device) {
-            if (alone && ran_dry(o)) {
-                g_queued.erase(g_queued.begin() + (std::ptrdiff_t)i--);
-                continue;
-            }
-            if (alone)
-                h->company = kRemembered;
-            o->company = kRemembered;
-            alone = false;
-            break;   // the first one in flight is enough, and it is told
+    for (size_t i = 0; i < g_flights.size();) {
+        Flight &o = *g_flights[i];
+        if (&o == &f || o.device != f.device) {
+            ++i;
+        } else if (landed(o)) {
+            g_flights.erase(g_flights.begin() + (std::ptrdiff_t)i);
+        } else {   // the first one in flight is enough, and it is told
+            f.company = o.company = kRemembered;
+            return false;
         }
     }
-    if (!listed && std::find(g_queued.begin(), g_queued.end(), h) == g_queued.end())
-        g_queued.push_back(h);
-    return alone;
+    return true;
 }
 
-void sweeps_waited(muca_t h)
+void flight_started(Flight &f, cudaStream_t s, bool own)
 {
-    std::lock_guard<std::mutex> lock(g_queued_mutex);
-    g_queued.erase(std::remove(g_queued.begin(), g_queued.end(), h), g_queued.end());
+    std::lock_guard<std::mutex> lock(g_flights_mutex);
+    if (own) {
+        f.ask = s;
+    } else {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
+            cudaGetLastError();
+            return;
+        }
+        if (capture != cudaStreamCaptureStatusNone)   // nothing runs yet
+            return;
+        const RelaxedCapture relaxed;
+        if (!relaxed.set || (!f.swept && cudaEventCreateWithFlags(&f.swept, cudaEventDisableTiming) != cudaSuccess) ||
+            cudaEventRecord(f.swept, s) != cudaSuccess) {
+            cudaGetLastError();
+            return;
+        }
+        f.ask = nullptr;
+    }
+    if (std::find(g_flights.begin(), g_flights.end(), &f) == g_flights.end())
+        g_flights.push_back(&f);
+}
+
+void flight_over(Flight &f)
+{
+    std::lock_guard<std::mutex> lock(g_flights_mutex);
+    g_flights.erase(std::remove(g_flights.begin(), g_flights.end(), &f), g_flights.end());
+}
+
+Flight::~Flight()
+{
+    flight_over(*this);
+    if (swept)
+        cudaEventDestroy(swept);
 }
 
 cudaError_t wait_stream(muca_t h)
 {
     const cudaError_t err = cudaStreamSynchronize(h->stream);
     if (err == cudaSuccess)
-        sweeps_waited(h);
+        flight_over(h->flight);
     return err;
 }
 
@@ -196,17 +225,18 @@ int run_attempts(muca_t h, uint64_t n, bool record, const uint32_t *skip)
     const uint64_t cap = record ? max_recorded_attempts(h->wpb) : UINT64_MAX;
     if (n == 0)
         return MUCA_OK;
-    const bool alone = sweeps_queued(h);
+    const bool alone = device_alone(h->flight);
     while (n > 0) {
         const uint64_t chunk = std::min(n, cap);
         const muca::SweepArgs a = sweep_args(h, chunk, skip);
         if (h->order == MUCA_ORDER_RANDOM)
             MUCA_CUDA(muca::launch_random_sweep(a, h->wpb, record, h->stream), "random-order sweep launch");
         else
-            MUCA_CUDA(muca::launch_sweep(a, h->wpb, alone, record, h->stream), "sweep launch");
+            MUCA_CUDA(muca::launch_sweep(a, h->wpb, alone, record, h->stream, &h->form), "sweep launch");
         h->t += chunk;
         n -= chunk;
     }
+    flight_started(h->flight, h->stream, h->stream == h->own_stream);
     return MUCA_OK;
 }
 
@@ -219,7 +249,8 @@ int run_therm_record(muca_t h, uint64_t n_therm, uint64_t n_record, const uint32
     }
     muca::SweepArgs a = sweep_args(h, n_record, skip);
     a.n_therm = n_therm;
-    MUCA_CUDA(muca::launch_sweep(a, h->wpb, sweeps_queued(h), true, h->stream), "sweep launch");
+    MUCA_CUDA(muca::launch_sweep(a, h->wpb, device_alone(h->flight), true, h->stream, &h->form), "sweep launch");
+    flight_started(h->flight, h->stream, h->stream == h->own_stream);
     h->t += n_therm + n_record;
     return MUCA_OK;
 }
@@ -526,7 +557,7 @@ int muca_create_ex(const muca_options *opt, muca_t *out)
     if (err != cudaSuccess)
         return cleanup(cuda_fail(err, "stream create"));
     h->stream = h->own_stream;
-    err = cudaGetDevice(&h->device);
+    err = cudaGetDevice(&h->flight.device);
     if (err != cudaSuccess)
         return cleanup(cuda_fail(err, "device query"));
     err = cudaEventCreateWithFlags(&h->table_copied, cudaEventDisableTiming);
@@ -579,7 +610,7 @@ int muca_destroy(muca_t h)
         return MUCA_OK;
     if (h->stream)
         cudaStreamSynchronize(h->stream);
-    sweeps_waited(h);
+    flight_over(h->flight);
     device_free(h->alloc, h->block);
     device_free(h->alloc, h->iter_block);
     if (h->h_iter)
@@ -1028,5 +1059,9 @@ int muca_philox(const uint32_t *ctr, const uint32_t key[2], size_t n, uint32_t *
 }
 
 const char *muca_last_error(void) { return g_last_error.c_str(); }
+
+// For tests, not part of muca.h: the form of the instance's last sweep launch, as the chain
+// warps per block of the paired kernel, 0 for loads two attempts ahead, -1 for direct loads.
+int32_t muca_testing_form(muca_t h) { return h->form.chains > 0 ? h->form.chains : h->form.ahead ? 0 : -1; }
 
 }  // extern "C"

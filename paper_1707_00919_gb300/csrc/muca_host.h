@@ -60,6 +60,26 @@ constexpr size_t kEnergyStageBytes = 256 * 1024;
 // shared histogram bins cannot overflow (each walker adds one count per attempt).
 inline uint64_t max_recorded_attempts(int wpb) { return 0xFFFFFFFFull / (uint64_t)std::max(wpb, 256); }
 
+// Sweeps queued on a device and perhaps still running, so that a launch knows whether it has
+// the device to itself (launch_sweep's form; results do not depend on it).  What says that
+// they have ended is their stream, where it is the library's own and outlives the flight,
+// else an event behind them: a caller's stream may be gone or under capture when another
+// instance asks, and may run the caller's own work.
+struct Flight {
+    int device = 0;
+    int company = 0;               // launches for which it is taken to overlap others
+    cudaStream_t ask = nullptr;    // null: ask `swept`
+    cudaEvent_t swept = nullptr;
+    ~Flight();
+};
+// Before a launch: true if no other flight of the device has sweeps running, or had some
+// together with f in the last few launches (who queues several in turn does so again).
+bool device_alone(Flight &f);
+// Behind a launch on s.
+void flight_started(Flight &f, cudaStream_t s, bool own);
+// The host has waited for them.
+void flight_over(Flight &f);
+
 // State of the weight iteration carried from one iteration to the next (Sec. 3):
 // extent and range of the energies visited in the previous iteration, whether the whole
 // range had been covered, and the previous N_updates.
@@ -76,8 +96,8 @@ struct muca_s {
     uint64_t seed = 0;
     int32_t layout = MUCA_LAYOUT_INT8;
     int32_t wpb = 64;
-    int device = 0;
-    int company = 0;                 // launches for which its sweeps are taken to overlap others (sweeps_queued)
+    muca_host::Flight flight;        // its sweeps, while the host has not seen their end
+    muca::SweepForm form{};          // of the last sweep launch
     muca_host::Allocator alloc;
     cudaStream_t own_stream = nullptr;
     cudaStream_t stream = nullptr;
@@ -119,14 +139,6 @@ void build_table(int32_t L, const std::vector<double> &lnW, uint32_t *T);
 int upload_table(muca_t h, bool zero_hist = false);
 int check_device_error(muca_t h);
 int sync_and_check(muca_t h);
-// Which instances have sweeps that the host has not waited for, so that a launch knows
-// whether it has the device to itself (launch_sweep's form; results do not depend on it).
-// sweeps_queued notes that h is about to launch one and returns true if no other instance
-// of the device has one in flight, or had one together with h in the last few launches (who
-// queues several instances in turn does so again); sweeps_waited notes that h's stream has
-// been waited for.
-bool sweeps_queued(muca_t h);
-void sweeps_waited(muca_t h);
 // Waits for the instance's stream.
 cudaError_t wait_stream(muca_t h);
 int run_attempts(muca_t h, uint64_t n, bool record, const uint32_t *skip = nullptr);

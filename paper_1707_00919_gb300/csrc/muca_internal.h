@@ -189,9 +189,11 @@ size_t launch_smem_bytes(int L, int walkers_per_block, bool guard = false, int s
 
 // Runs a.n_therm thermalization attempts from a.t0 (recording launches only; may be 0),
 // then a.n attempts of every walker: one launch unless the range crosses a step of counter
-// word 1 (every 2^34 attempts).  alone: no other sweep of the process is in flight on the
-// device, so that the launch may take more SMs than its walkers fill (SweepForm).
-cudaError_t launch_sweep(const SweepArgs &a, int walkers_per_block, bool alone, bool record, cudaStream_t s);
+// word 1 (every 2^34 attempts).  alone: no other sweep that the library knows of is in flight
+// on the device, so that the launch may take more SMs than its walkers fill.  *form receives
+// the form taken.
+cudaError_t launch_sweep(const SweepArgs &a, int walkers_per_block, bool alone, bool record, cudaStream_t s,
+                         SweepForm *form);
 
 // Runs attempts [t0, t0 + n) of every walker in random shared site order (muca_random.cu;
 // any L, any attempt range; the given block size, or a smaller one that fits shared

@@ -203,9 +203,9 @@ SweepForm sweep_form(const SweepArgs &a, int wpb, bool alone)
 }
 
 // Dispatches a launch to the kernel for L.
-cudaError_t launch_full(const SweepArgs &a, int wpb, bool alone, bool record, cudaStream_t s)
+cudaError_t launch_full(const SweepArgs &a, int wpb, bool alone, bool record, cudaStream_t s, SweepForm &form)
 {
-    const SweepForm form = sweep_form(a, wpb, alone);
+    form = sweep_form(a, wpb, alone);
     switch (a.L) {
     case 4: return launch_full_L4(a, wpb, form, record, s);
     case 8: return launch_full_L8(a, wpb, form, record, s);
@@ -260,7 +260,7 @@ size_t sweep_smem_limit()
     return (size_t)v;
 }
 
-cudaError_t launch_sweep(const SweepArgs &a, int wpb, bool alone, bool record, cudaStream_t s)
+cudaError_t launch_sweep(const SweepArgs &a, int wpb, bool alone, bool record, cudaStream_t s, SweepForm *form)
 {
     if (a.W == 0 || (a.n == 0 && a.n_therm == 0))
         return cudaSuccess;
@@ -269,16 +269,16 @@ cudaError_t launch_sweep(const SweepArgs &a, int wpb, bool alone, bool record, c
         // not one launch: the thermalization by itself
         part.n_therm = 0;
         part.n = a.n_therm;
-        const cudaError_t err = launch_sweep(part, wpb, alone, false, s);
+        const cudaError_t err = launch_sweep(part, wpb, alone, false, s, form);
         if (err != cudaSuccess)
             return err;
         part.t0 = a.t0 + a.n_therm;
         part.n = a.n;
-        return launch_sweep(part, wpb, alone, record, s);
+        return launch_sweep(part, wpb, alone, record, s, form);
     }
     for (uint64_t left = a.n; left > 0; left -= part.n, part.t0 += part.n) {
         part.n = a.n_therm > 0 ? left : same_word1(part.t0, left);
-        const cudaError_t err = launch_full(part, wpb, alone, record, s);
+        const cudaError_t err = launch_full(part, wpb, alone, record, s, *form);
         if (err != cudaSuccess)
             return err;
     }
