@@ -36,6 +36,7 @@ struct muca_batch_s {
     int grid = 0;
     cudaGraphExec_t exec = nullptr;       // one weight iteration of the current members
     uint64_t g_therm = 0, g_rec = 0;
+    Flight flight;                        // its launches, while the host has not seen their end
 };
 
 namespace {
@@ -270,6 +271,11 @@ int batch_run_iteration(muca_batch_t b, const std::vector<int32_t> &active, cons
             return rc;
     }
     const size_t nm = active.size();
+    // from here to the end the stream is not captured, so that it can be asked
+    struct Landing {
+        Flight &f;
+        ~Landing() { flight_over(f); }
+    } landing{b->flight};
     const uint64_t cap = max_recorded_attempts(256);
     bool chunked = false;
     for (size_t j = 0; j < nm; ++j)
@@ -289,6 +295,7 @@ int batch_run_iteration(muca_batch_t b, const std::vector<int32_t> &active, cons
     }
     if (!chunked) {
         MUCA_CUDA(cudaGraphLaunch(b->exec, b->stream), "batch iteration launch");
+        flight_started(b->flight, b->stream, true);
         MUCA_CUDA(cudaStreamSynchronize(b->stream), "batch synchronize");
     } else {
         MUCA_CUDA(cudaMemcpyAsync(b->d_args, b->h_args, sizeof(muca::SweepArgs) * 2 * nm, cudaMemcpyHostToDevice,
@@ -298,10 +305,12 @@ int batch_run_iteration(muca_batch_t b, const std::vector<int32_t> &active, cons
         MUCA_CUDA(muca::launch_batch(b->d_args, b->d_items, b->n_items, b->d_work, b->grid, b->smem_launch, false,
                                      b->stream),
                   "batched thermalization");
+        flight_started(b->flight, b->stream, true);
         for (uint64_t done = 0;;) {
             MUCA_CUDA(muca::launch_batch(b->d_args + nm, b->d_items, b->n_items, b->d_work, b->grid, b->smem_launch,
                                          true, b->stream),
                       "batched recording");
+            flight_started(b->flight, b->stream, true);
             done += cap;
             bool more = false;
             for (size_t j = 0; j < nm; ++j)
@@ -462,6 +471,7 @@ int muca_batch_create(const muca_t *instances, int32_t n, muca_batch_t *out)
         err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (err != cudaSuccess)
         return cleanup(cuda_fail(err, "multiprocessor count"));
+    b->flight.device = dev;
     const int occ = muca::batch_resident_blocks(b->smem_launch);
     if (occ < 1)
         return cleanup(fail(MUCA_EINVAL, "batched kernel does not fit an SM with %zu bytes of shared memory", b->smem));
@@ -581,6 +591,7 @@ int muca_batch_sweep(muca_batch_t b, uint64_t n_sweeps, int record)
         MUCA_CUDA(muca::launch_batch(b->d_args, b->d_items, b->n_items, b->d_work, b->grid, b->smem_launch, record != 0,
                                      b->stream),
                   "batched launch");
+        flight_started(b->flight, b->stream, false);
         n_sweeps -= chunk;
     }
     return MUCA_OK;

@@ -85,3 +85,33 @@ def test_members_of_a_batch_and_after_it(M):
             batch.sweep(1, record=False)
         c.sweep(1, record=False)   # closing the batch has waited
         assert paired(c)
+
+
+def test_batched_sweeps(M):
+    import torch
+    with M.Muca(32, 1024, 1) as a, M.Muca(32, 1024, 2) as b, M.Muca(32, 1024, 3) as c:
+        with M.Batch([a]) as batch:
+            batch.sweep(LONG, record=False)
+            b.sweep(1, record=False)
+            assert not paired(b)
+            torch.cuda.synchronize()
+            c.sweep(1, record=False)
+            assert paired(c)
+
+
+def test_batched_iteration_in_another_thread(M):
+    import threading
+    with M.Muca(32, 1024, 1) as a, M.Muca(32, 1024, 2) as b, M.Muca(32, 1024, 3) as c:
+        with M.Batch([a]) as batch:
+            params = M.make_params(therm_sweeps=LONG, sweeps_per_iter=1, max_iterations=1, flat_threshold=2.0)
+            t = threading.Thread(target=batch.iterate_until_flat, args=(params,))
+            t.start()
+            forms = []
+            while t.is_alive():
+                b.sweep(1, record=False)
+                b.synchronize()
+                forms.append(paired(b))
+            t.join()
+            assert not all(forms)   # the launches before the iteration's own may be
+            c.sweep(1, record=False)
+            assert paired(c)
