@@ -752,6 +752,13 @@ int muca_batch_sweep_noalloc(const muca_raw_instance *instances, int32_t n, uint
     MUCA_CUDA(muca::launch_batch_noalloc(descs, wpbs, prefix, n, smem, record != 0,
                                          static_cast<cudaStream_t>(cuda_stream)),
               "allocation-free batched sweep");
+    // calls do not overlap, so that a flight per device (kept to the end of the process) holds
+    static Flight *const flights = new (std::nothrow) Flight[muca::kNoAllocMaxDevices];
+    int dev = 0;
+    if (flights && cudaGetDevice(&dev) == cudaSuccess) {
+        flights[dev].device = dev;
+        flight_started(flights[dev], static_cast<cudaStream_t>(cuda_stream), false);
+    }
     return MUCA_OK;
 }
 

@@ -60,7 +60,7 @@ constexpr size_t kEnergyStageBytes = 256 * 1024;
 // shared histogram bins cannot overflow (each walker adds one count per attempt).
 inline uint64_t max_recorded_attempts(int wpb) { return 0xFFFFFFFFull / (uint64_t)std::max(wpb, 256); }
 
-// Sweeps of an instance or batch queued on a device and perhaps still running, so that a launch knows whether it has
+// Sweeps of an instance, a batch or allocation-free calls, queued on a device and perhaps still running, so that a launch knows whether it has
 // the device to itself (launch_sweep's form; results do not depend on it).  What says that
 // they have ended is their stream, where it is the library's own and outlives the flight,
 // else an event behind them: a caller's stream may be gone or under capture when another

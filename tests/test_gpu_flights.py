@@ -115,3 +115,23 @@ def test_batched_iteration_in_another_thread(M):
             assert not all(forms)   # the launches before the iteration's own may be
             c.sweep(1, record=False)
             assert paired(c)
+
+
+def test_allocation_free_sweeps(M):
+    import torch
+    from paper_1707_00919_gb300 import _lib as C
+    L, W, st = 32, 1024, torch.cuda.Stream()
+    N = L * L
+    zeros = lambda n, t: torch.zeros(n, dtype=t, device="cuda")
+    bufs = (torch.ones(N * W, dtype=torch.int8, device="cuda"), zeros(W, torch.int32), zeros(5 * (N + 1), torch.int32),
+            zeros(N + 1, torch.int64), zeros(1, torch.int32))   # all spins up, no flip accepted
+    r = C.muca_raw_instance(L, 0, W, 1, 0, *(t.data_ptr() for t in bufs))
+    torch.cuda.synchronize()
+    with M.Muca(L, W, 2) as b, M.Muca(L, W, 3) as c:
+        M.muca_batch_sweep_noalloc([r], LONG // 2, False, st.cuda_stream)
+        b.sweep(1, record=False)
+        assert not paired(b)
+        st.synchronize()
+        c.sweep(1, record=False)
+        assert paired(c)
+    assert int(bufs[4].item()) == 0
