@@ -216,23 +216,25 @@ cudaError_t launch_unpack(int32_t L, int32_t layout, int64_t W, const void *latt
 cudaError_t launch_philox(const uint32_t *ctr, uint32_t k0, uint32_t k1, size_t n, uint32_t *out,
                           cudaStream_t s);
 
-// Kernels of one L each (muca_full_L.cu): launch over any attempt range in the given form.
-cudaError_t launch_full_L4(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
-cudaError_t launch_full_L8(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
-cudaError_t launch_full_L12(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
-cudaError_t launch_full_L16(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
-cudaError_t launch_full_L20(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
-cudaError_t launch_full_L24(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
-cudaError_t launch_full_L28(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
-cudaError_t launch_full_L32(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
-cudaError_t launch_full_L36(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
-cudaError_t launch_full_L40(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
-cudaError_t launch_full_L44(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
-cudaError_t launch_full_L48(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
-cudaError_t launch_full_L52(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
-cudaError_t launch_full_L56(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
-cudaError_t launch_full_L60(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
-cudaError_t launch_full_L64(const SweepArgs &a, int wpb, SweepForm form, bool record, cudaStream_t s);
+// Kernels of one L each (muca_full_L.cu): launch over any attempt range in the given form;
+// direct loads (not ahead) only if an SM holds more than eight warps at once, else form.ahead
+// is set.
+cudaError_t launch_full_L4(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
+cudaError_t launch_full_L8(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
+cudaError_t launch_full_L12(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
+cudaError_t launch_full_L16(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
+cudaError_t launch_full_L20(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
+cudaError_t launch_full_L24(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
+cudaError_t launch_full_L28(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
+cudaError_t launch_full_L32(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
+cudaError_t launch_full_L36(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
+cudaError_t launch_full_L40(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
+cudaError_t launch_full_L44(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
+cudaError_t launch_full_L48(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
+cudaError_t launch_full_L52(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
+cudaError_t launch_full_L56(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
+cudaError_t launch_full_L60(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
+cudaError_t launch_full_L64(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
 
 // Blocks of the sweep kernel for this L, layout and block size that one SM holds at once
 // by the sizing rule (0 if the configuration does not fit).

@@ -184,8 +184,9 @@ __global__ void philox_kernel(const uint32_t *ctr, uint32_t k0, uint32_t k1, siz
 // (when sweeps of other instances run, it would take SMs from them for less throughput:
 // eight instances of L = 32 with 4096 walkers, all queued, 1661 us per 20 sweeps with it
 // against 955).  Up to eight, two per sub-partition: the two-ahead loads.  More than that
-// resident at once: direct loads, whose latency the other warps cover.
-SweepForm sweep_form(const SweepArgs &a, int wpb, bool alone)
+// resident at once: direct loads, whose latency the other warps cover (how many the kernel's
+// blocks leave resident is looked at where it is launched, muca_full.cuh).
+SweepForm sweep_form(const SweepArgs &a, bool alone)
 {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -199,13 +200,13 @@ SweepForm sweep_form(const SweepArgs &a, int wpb, bool alone)
         const bool two = warps > sms || (a.L >= 52 && warps > 1);
         return {two ? 2 : 1, true};
     }
-    return {0, warps <= 8 * (int64_t)sms || resident_blocks(a.L, a.layout, wpb) * (wpb / 32) <= 8};
+    return {0, warps <= 8 * (int64_t)sms};
 }
 
 // Dispatches a launch to the kernel for L.
 cudaError_t launch_full(const SweepArgs &a, int wpb, bool alone, bool record, cudaStream_t s, SweepForm &form)
 {
-    form = sweep_form(a, wpb, alone);
+    form = sweep_form(a, alone);
     switch (a.L) {
     case 4: return launch_full_L4(a, wpb, form, record, s);
     case 8: return launch_full_L8(a, wpb, form, record, s);
