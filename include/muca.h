@@ -75,7 +75,7 @@ extern "C" {
 
 /* walkers_per_block value of muca_create_ex that times every block size from 32 to 256
  * (two recorded sweeps each on a temporary instance) and keeps the fastest.  0 picks
- * one from the kernel's occupancy without timing. */
+ * one without timing, from the resident blocks as muca_optimal_walkers counts them. */
 #define MUCA_WPB_TUNE (-1)
 
 /* n_walkers value of muca_create / muca_create_ex that asks for the walker count of
@@ -163,9 +163,14 @@ int muca_create_ex(const muca_options *opt, muca_t *out);
  * flip lies where every multiprocessor holds its maximal number of resident blocks, and
  * the program uses that count when W is not given).  For lattice side L and layout
  * (MUCA_LAYOUT_INT8 or MUCA_LAYOUT_PACKED) on the current device: the block size whose
- * resident blocks per SM (whole-sweep kernel, shared memory and registers) hold the
- * most walkers, ties to the larger block; *n_walkers = SMs x resident blocks x block
- * size, *walkers_per_block (may be NULL) = that block size.  Nothing is allocated.
+ * resident blocks per SM hold the most walkers, ties to the larger block; *n_walkers =
+ * SMs x resident blocks x block size, *walkers_per_block (may be NULL) = that block size.
+ * The resident blocks are counted with a fixed register and shared-memory demand per L and
+ * layout, so that the count, and with it the chains of an instance created without one,
+ * stays the same from one version of the kernels to the next.  At L = 4, 12, 20, 28, 40, 44
+ * and, with MUCA_LAYOUT_INT8, 8 the kernels hold fewer at once (512, 640, 512, 384, 384, 320
+ * and 512 walkers per SM where the rule counts 2048, 2048, 1792, 1120, 448, 384 and 768): such
+ * an instance runs in two to four waves.  Nothing is allocated.
  * Errors: MUCA_EINVAL (L as in muca_create, other layout, n_walkers NULL, no block size
  * fits), MUCA_ECUDA. */
 int muca_optimal_walkers(int32_t L, int32_t layout, int64_t *n_walkers, int32_t *walkers_per_block);

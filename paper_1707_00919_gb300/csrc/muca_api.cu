@@ -315,10 +315,12 @@ bool get(FILE *f, T *v, size_t n)
     return std::fread(v, sizeof(T), n, f) == n;
 }
 
-// Block size for L, layout and W by occupancy: the makespan of a launch is set by the
+// Block size for L, layout and W by the occupancy of the sizing rule: the makespan of a launch is set by the
 // most loaded SM sub-partition (one walker per thread, one warp per 32 walkers), so the
 // cost of a block size is waves x warps per sub-partition in a full wave; ties go to
-// the larger block.
+// the larger block.  (With the kernels' own occupancy some counts would do better, L = 44 with
+// 40 000 walkers 119 us per sweep instead of 162, and others worse, L = 20 with 87 986 walkers
+// 46.4 instead of 40.8, L = 28 with 90 000 walkers 95 instead of 87: the last wave is not a full one.)
 int default_walkers_per_block(int32_t L, int32_t layout, int64_t W)
 {
     int dev = 0, sms = 0;

@@ -179,7 +179,7 @@ struct BatchItem {
 constexpr int kBatchThreads = 256;   // threads per block of the batched kernel
 
 // Shared memory bytes that the sizing rule counts for an L without a register count of its
-// own (bit rows, thresholds and counts).
+// own (bit rows, thresholds and counts; not what the kernel takes, launch_smem_bytes).
 size_t sizing_smem_bytes(int L, int walkers_per_block);
 
 // Shared memory bytes of the sweep kernel's table and rows, by which block sizes are
@@ -236,8 +236,8 @@ cudaError_t launch_full_L56(const SweepArgs &a, int wpb, SweepForm &form, bool r
 cudaError_t launch_full_L60(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
 cudaError_t launch_full_L64(const SweepArgs &a, int wpb, SweepForm &form, bool record, cudaStream_t s);
 
-// Blocks of the sweep kernel for this L, layout and block size that one SM holds at once
-// by the sizing rule (0 if the configuration does not fit).
+// Blocks for this L, layout and block size that one SM holds at once by the sizing rule of the
+// default walker count and block size (0 if the configuration does not fit).
 int resident_blocks(int L, int layout, int walkers_per_block);
 
 // Batched persistent kernel: allows `smem` bytes of dynamic shared memory, reports how

@@ -352,11 +352,13 @@ cudaError_t launch_philox(const uint32_t *ctr, uint32_t k0, uint32_t k1, size_t 
     return cudaGetLastError();
 }
 
-// Registers per thread that the sizing rule counts with, by L and layout; 0 where L is
-// bounded by shared memory and threads alone.  The default block size, the walker count
-// of full occupancy and with it the chains of an instance created without an explicit
-// count follow from this rule, so it is fixed and does not move with the register
-// allocation of the sweep kernels (which stay below it or within 10 % of it).
+// Registers per thread that the sizing rule counts with, by L and layout; 0 where it counts
+// bit rows, six words per table row and threads alone.  The walker count of full occupancy
+// and with it the chains of an instance created without an explicit count, and the default
+// block size, follow from this rule, so it is fixed and does not move with the sweep kernels.
+// It is theirs at L = 16, 24, 32, 36, 48, 52, 56, 60 and 64; at the other sizes they need more
+// (100 registers at L = 8, 106 at L = 4) and fewer walkers fit an SM than it says (muca.h).
+// What a launch takes for granted is asked of its kernel (muca_full.cuh).
 static int sizing_registers(int L, int layout)
 {
     const bool packed = layout == MUCA_LAYOUT_PACKED;

@@ -30,3 +30,14 @@ def test_form_by_resident_warps(M, L, wpb, form):
         m.attempts(4, record=False)
         assert C.load().muca_testing_form(m._h) == form
         assert (m.get_energies() >= 0).all()
+
+
+@pytest.mark.parametrize("layout", [0, 1])
+def test_default_counts_are_fixed(M, layout):
+    """The walkers per SM of the default count, which decides the chains of an instance created
+    without one."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    counts = {4: 2048, 8: 512 if layout else 768, 12: 2048, 16: 640, 20: 1792, 24: 512, 28: 1120, 32: 320, 36: 512,
+              40: 448, 44: 384, 48: 256, 52: 256, 56: 256, 60: 256, 64: 224}
+    assert {L: M.muca_optimal_walkers(L, layout)[0] // sms for L in counts} == counts
