@@ -1,5 +1,7 @@
 // muca_batch.cu - the batched persistent kernel: one launch advances many instances of
 // uneven L and walker count (work list and counter in library memory).
+#include <mutex>
+
 #include "muca_device.cuh"
 
 namespace muca {
@@ -75,7 +77,20 @@ __global__ void __launch_bounds__(kBatchThreads, 1) batch_kernel(const SweepArgs
 
 cudaError_t configure_batch(size_t smem)
 {
-    return cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the bound is the kernel's, for all batches alive: one that needs less leaves it
+    static std::mutex mutex;
+    static size_t bound[64] = {};
+    int dev = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess)
+        return err;
+    const std::lock_guard<std::mutex> lock(mutex);
+    if (dev < 64 && smem <= bound[dev])
+        return cudaSuccess;
+    err = cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err == cudaSuccess && dev < 64)
+        bound[dev] = smem;
+    return err;
 }
 
 int batch_resident_blocks(size_t smem)
