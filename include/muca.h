@@ -403,8 +403,8 @@ typedef struct muca_batch_s *muca_batch_t;
 /* Groups n existing instances.  The batch does not own them; while it exists their
  * work runs on the batch's stream (ordered with batch launches); muca_batch_destroy
  * gives each instance its stream back.  Allocates the launch descriptors, the work list
- * and the work counters on the device.  Errors: MUCA_EINVAL (NULL, duplicates, L
- * without a whole-sweep kernel), MUCA_ENOMEM, MUCA_ECUDA. */
+ * and the work counters on the device.  Errors: MUCA_EINVAL (NULL, duplicates, another L),
+ * MUCA_ENOMEM, MUCA_ECUDA. */
 int muca_batch_create(const muca_t *instances, int32_t n, muca_batch_t *out);
 int muca_batch_destroy(muca_batch_t b);
 

@@ -31,8 +31,7 @@ struct muca_batch_s {
     int32_t n_items = 0;                  // items of the current member set
     std::vector<int32_t> members;         // instances in the current work list
     uint64_t longest = 0;                 // longest chain that the work list was made for
-    size_t smem = 0;                      // of the largest member's table and rows
-    size_t smem_launch = 0;               // of a launch
+    size_t smem = 0;                      // of a launch: the largest member's table and rows
     int grid = 0;
     cudaGraphExec_t exec = nullptr;       // one weight iteration of the current members
     uint64_t g_therm = 0, g_rec = 0;
@@ -189,7 +188,7 @@ int build_graph(muca_batch_t b)
     if (err == cudaSuccess)
         err = muca::launch_batch_tables(b->d_jobs, (int32_t)nm, b->bins, b->stream);
     if (err == cudaSuccess)
-        err = muca::launch_batch(b->d_args + nm, b->d_items, b->n_items, b->d_work, b->grid, b->smem_launch, true,
+        err = muca::launch_batch(b->d_args + nm, b->d_items, b->n_items, b->d_work, b->grid, b->smem, true,
                                  b->stream);
     if (err == cudaSuccess)
         err = muca::launch_batch_read(b->d_jobs, (int32_t)nm, b->bins, b->stream);
@@ -302,12 +301,12 @@ int batch_run_iteration(muca_batch_t b, const std::vector<int32_t> &active, cons
                                   b->stream),
                   "batch descriptor upload");
         MUCA_CUDA(muca::launch_batch_tables(b->d_jobs, (int32_t)nm, b->bins, b->stream), "batch tables");
-        MUCA_CUDA(muca::launch_batch(b->d_args, b->d_items, b->n_items, b->d_work, b->grid, b->smem_launch, false,
+        MUCA_CUDA(muca::launch_batch(b->d_args, b->d_items, b->n_items, b->d_work, b->grid, b->smem, false,
                                      b->stream),
                   "batched thermalization");
         flight_started(b->flight, b->stream, true);
         for (uint64_t done = 0;;) {
-            MUCA_CUDA(muca::launch_batch(b->d_args + nm, b->d_items, b->n_items, b->d_work, b->grid, b->smem_launch,
+            MUCA_CUDA(muca::launch_batch(b->d_args + nm, b->d_items, b->n_items, b->d_work, b->grid, b->smem,
                                          true, b->stream),
                       "batched recording");
             flight_started(b->flight, b->stream, true);
@@ -422,8 +421,7 @@ int muca_batch_create(const muca_t *instances, int32_t n, muca_batch_t *out)
         if (!instances[i])
             return fail(MUCA_EINVAL, "instance %d is NULL", i);
         if (!batchable_L(instances[i]->L))
-            return fail(MUCA_EINVAL, "instance %d: L = %d has no whole-sweep kernel (8, 16, 24, 32, 48, 64)", i,
-                        instances[i]->L);
+            return fail(MUCA_EINVAL, "instance %d: L = %d not in {8, 16, 24, 32, 48, 64}", i, instances[i]->L);
         if (instances[i]->order != MUCA_ORDER_TYPEWRITER)
             return fail(MUCA_EINVAL, "instance %d: the batched kernel runs typewriter order only", i);
         if (instances[i]->reducer)
@@ -452,8 +450,7 @@ int muca_batch_create(const muca_t *instances, int32_t n, muca_batch_t *out)
         while (wpb > 32 && muca::full_smem_bytes(h->L, wpb, true, false, stride) > limit)
             wpb -= 32;
         b->item_wpb.push_back(wpb);
-        b->smem = std::max(b->smem, muca::full_smem_bytes(h->L, wpb, true, false, stride));
-        b->smem_launch = std::max(b->smem_launch, muca::launch_smem_bytes(h->L, wpb, false, stride));
+        b->smem = std::max(b->smem, muca::launch_smem_bytes(h->L, wpb, false, stride));
         const int small = std::min(wpb, kSmallItem);
         items += (size_t)((h->W + small - 1) / small);
     }
@@ -462,7 +459,7 @@ int muca_batch_create(const muca_t *instances, int32_t n, muca_batch_t *out)
     if (err == cudaSuccess)
         err = cudaEventCreateWithFlags(&b->staged, cudaEventDisableTiming);
     if (err == cudaSuccess)
-        err = muca::configure_batch(b->smem_launch);
+        err = muca::configure_batch(b->smem);
     if (err != cudaSuccess)
         return cleanup(cuda_fail(err, "batch set-up"));
     int dev = 0, sms = 0;
@@ -472,7 +469,7 @@ int muca_batch_create(const muca_t *instances, int32_t n, muca_batch_t *out)
     if (err != cudaSuccess)
         return cleanup(cuda_fail(err, "multiprocessor count"));
     b->flight.device = dev;
-    const int occ = muca::batch_resident_blocks(b->smem_launch);
+    const int occ = muca::batch_resident_blocks(b->smem);
     if (occ < 1)
         return cleanup(fail(MUCA_EINVAL, "batched kernel does not fit an SM with %zu bytes of shared memory", b->smem));
     b->grid = sms * occ;
@@ -588,7 +585,7 @@ int muca_batch_sweep(muca_batch_t b, uint64_t n_sweeps, int record)
                                   cudaMemcpyHostToDevice, b->stream),
                   "batch descriptor upload");
         MUCA_CUDA(cudaEventRecord(b->staged, b->stream), "batch upload event");
-        MUCA_CUDA(muca::launch_batch(b->d_args, b->d_items, b->n_items, b->d_work, b->grid, b->smem_launch, record != 0,
+        MUCA_CUDA(muca::launch_batch(b->d_args, b->d_items, b->n_items, b->d_work, b->grid, b->smem, record != 0,
                                      b->stream),
                   "batched launch");
         flight_started(b->flight, b->stream, false);

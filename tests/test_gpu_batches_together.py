@@ -36,3 +36,13 @@ def test_a_smaller_batch_leaves_the_larger_one_usable(M):
         big.close()
         small.close()
     assert all(np.array_equal(x, y) for x, y in zip(*out))
+
+
+@pytest.mark.parametrize("L,W", [(8, 64), (32, 700), (64, 300)])
+def test_info_reports_the_shared_memory_of_a_launch(M, L, W):
+    """Table (a row of zeros behind the energies; 24-byte rows at L = 64, else 28) and the rows
+    of a block's walkers."""
+    with M.Muca(L, W, 1) as m, M.Batch([m]) as b:
+        table = -(-(L * L + 2) * (24 if L == 64 else 28) // 16) * 16
+        rows = L * (4 * ((L + 7) // 8) if L <= 32 else 8)
+        assert b.info()[2] == table + rows * 256
