@@ -1062,8 +1062,10 @@ int muca_philox(const uint32_t *ctr, const uint32_t key[2], size_t n, uint32_t *
 
 const char *muca_last_error(void) { return g_last_error.c_str(); }
 
-// For tests, not part of muca.h: the form of the instance's last sweep launch, as the chain
-// warps per block of the paired kernel, 0 for loads two attempts ahead, -1 for direct loads.
+// For tests, not part of muca.h: whether the waits of the instance's paired kernels run out at
+// once (L = 8 and 32), and the form of its last sweep launch, as the chain warps per block of the paired
+// kernel, 0 for loads two attempts ahead, -1 for direct loads.
+void muca_testing_no_waits(muca_t h, int32_t on) { h->form.no_waits = on != 0; }
 int32_t muca_testing_form(muca_t h) { return h->form.chains > 0 ? h->form.chains : h->form.ahead ? 0 : -1; }
 
 }  // extern "C"

@@ -77,6 +77,9 @@ cudaError_t MUCA_CAT(launch_full_L, MUCA_L)(const SweepArgs &a, int wpb, SweepFo
 {
     using Ahead = AttemptStream<MUCA_L, kTableStride, (MUCA_L <= 32 ? 1 : 0)>;
     using Direct = DirectStream<MUCA_L, kTableStride>;
+    if constexpr (MUCA_L == 8 || MUCA_L == 32)   // for tests
+        if (form.chains > 0 && form.no_waits)
+            return launch_pair_t<MUCA_L, 0>(a, form.chains, record, s);
     if (form.chains > 0)
         return launch_pair_t<MUCA_L>(a, form.chains, record, s);
     // the walkers are many, but an SM may hold two warps per sub-partition at a time all the

@@ -118,6 +118,7 @@ cudaError_t allow_smem(Kernel kern, std::atomic<uint64_t> &done)
 struct SweepForm {
     int32_t chains;
     bool ahead;
+    bool no_waits = false;   // for tests, L = 8 and 32: every wait of the paired kernel runs out at once
 };
 
 // Waits between the warps of the paired kernel: tries of at most 20 us each before a wait

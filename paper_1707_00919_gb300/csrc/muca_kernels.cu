@@ -206,7 +206,9 @@ SweepForm sweep_form(const SweepArgs &a, bool alone)
 // Dispatches a launch to the kernel for L.
 cudaError_t launch_full(const SweepArgs &a, int wpb, bool alone, bool record, cudaStream_t s, SweepForm &form)
 {
+    const bool no_waits = form.no_waits;
     form = sweep_form(a, alone);
+    form.no_waits = no_waits;
     switch (a.L) {
     case 4: return launch_full_L4(a, wpb, form, record, s);
     case 8: return launch_full_L8(a, wpb, form, record, s);

@@ -27,12 +27,13 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
     asm volatile("mbarrier.arrive.shared.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// Waits for the phase of the given parity, kPairWaitTries tries of at most 20 us each;
-// false on expiry.
+// Waits for the phase of the given parity, TRIES times at most 20 us; false on expiry.  (A
+// number of tries that comes with the launch made the kernel 2 % slower.)
+template <uint32_t TRIES>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
 {
 #pragma unroll 1
-    for (uint32_t i = 0; i < kPairWaitTries; ++i) {
+    for (uint32_t i = 0; i < TRIES; ++i) {
         uint32_t done;
         asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
                      : "=r"(done)
@@ -47,7 +48,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
 // One chain warp's ring: two slots of a chunk of rows each, 16 bytes per lane and Philox
 // block, with a full and an empty barrier per slot.  Chunks are counted over the launch
 // (c), so that both sides agree on slot and phase.
-template <int L>
+template <int L, uint32_t TRIES>
 struct PairRing {
     static constexpr int kRows = L < 128 ? 128 / L : 1;             // rows per chunk
     static constexpr int kTogether = 4;                             // blocks drawn together
@@ -72,7 +73,7 @@ struct PairRing {
         for (uint64_t left = nrows; left > 0;) {
             const int rows = left < (uint64_t)kRows ? (int)left : kRows;
             if ((int)(c & (uint32_t)(gens - 1)) == j) {
-                ok = ok && mbar_wait(empty(), ((c >> 1) & 1u) ^ 1u);
+                ok = ok && mbar_wait<TRIES>(empty(), ((c >> 1) & 1u) ^ 1u);
                 uint32_t at = slot();
                 const int nb = rows * (L / 4);
 #pragma unroll 1
@@ -145,9 +146,9 @@ struct RingSource {
 };
 
 // Whole rows of a chain warp (see stream_rows) with the words of its ring.
-template <int L, int STRIDE>
-__device__ __forceinline__ uint32_t ring_rows(const SmemRows<L> &rows, uint32_t E, int y, uint64_t nrows, PairRing<L> &ring,
-                                              int lane)
+template <int L, int STRIDE, uint32_t TRIES>
+__device__ __forceinline__ uint32_t ring_rows(const SmemRows<L> &rows, uint32_t E, int y, uint64_t nrows,
+                                              PairRing<L, TRIES> &ring, int lane)
 {
     constexpr int NW = row_words(L);
     uint32_t U[NW], C[NW], D[NW];
@@ -158,8 +159,8 @@ __device__ __forceinline__ uint32_t ring_rows(const SmemRows<L> &rows, uint32_t 
     st.start(U, C, D, E);
 #pragma unroll 1
     for (uint64_t left = nrows; left > 0;) {
-        const int n = left < (uint64_t)PairRing<L>::kRows ? (int)left : PairRing<L>::kRows;
-        ring.ok = ring.ok && mbar_wait(ring.full(), (ring.c >> 1) & 1u);
+        const int n = left < (uint64_t)ring.kRows ? (int)left : ring.kRows;
+        ring.ok = ring.ok && mbar_wait<TRIES>(ring.full(), (ring.c >> 1) & 1u);
         RingSource src;
         src.at = ring.slot();
         src.load();
@@ -189,7 +190,7 @@ __device__ __forceinline__ uint32_t ring_rows(const SmemRows<L> &rows, uint32_t 
 
 // Blocks of `chains` chain warps (32 walkers each), then `gens` (1 or 2) generator warps
 // per chain warp.
-template <int L>
+template <int L, uint32_t TRIES>
 __global__ void __launch_bounds__(kPairMaxThreads, 1) pair_kernel(const SweepArgs a, const __grid_constant__ LaunchPlan plan,
                                                                   const int chains, const int gens, const bool record)
 {
@@ -204,9 +205,9 @@ __global__ void __launch_bounds__(kPairMaxThreads, 1) pair_kernel(const SweepArg
     const int pair = chain ? warp : (warp - chains) % chains;
     uint32_t *sTab = reinterpret_cast<uint32_t *>(smem);
     unsigned char *sRows = smem + align_up((size_t)(NB + 1) * STRIDE * 4, 16);
-    unsigned char *sRing = sRows + (size_t)(32 * chains) * SmemRows<L>::bytes_per_walker() + (size_t)pair * PairRing<L>::bytes();
+    unsigned char *sRing = sRows + (size_t)(32 * chains) * SmemRows<L>::bytes_per_walker() + (size_t)pair * PairRing<L, TRIES>::bytes();
     const SmemRows<L> rows{sRows, 32 * chains, 32 * pair + lane};
-    PairRing<L> ring;
+    PairRing<L, TRIES> ring;
     ring.bars = (uint32_t)__cvta_generic_to_shared(sRing);
     ring.base = ring.bars + 32u + 16u * (uint32_t)lane;
     const int64_t w = ((int64_t)blockIdx.x * chains + pair) * 32 + lane;
@@ -249,7 +250,7 @@ __global__ void __launch_bounds__(kPairMaxThreads, 1) pair_kernel(const SweepArg
                 for (int part = 0; part < 3; ++part) {
                     if (part == 1) {
                         if (p.rows > 0)
-                            E = ring_rows<L, STRIDE>(rows, E, p.y1, p.rows, ring, lane);
+                            E = ring_rows<L, STRIDE, TRIES>(rows, E, p.y1, p.rows, ring, lane);
                     } else {
                         const int x0 = part == 0 ? p.x0 : 0, x1 = part == 0 ? p.x0_end : p.tail;
                         if (x0 < x1)
@@ -285,13 +286,13 @@ __global__ void __launch_bounds__(kPairMaxThreads, 1) pair_kernel(const SweepArg
         a.energy[w] = e;
 }
 
-template <int L>
+template <int L, uint32_t TRIES = kPairWaitTries>
 cudaError_t launch_pair_t(const SweepArgs &a, int chains, bool record, cudaStream_t s)
 {
     const size_t smem = align_up((size_t)(L * L + 2) * kTableStride * 4, 16) +
-                        (size_t)chains * (32 * SmemRows<L>::bytes_per_walker() + PairRing<L>::bytes());
+                        (size_t)chains * (32 * SmemRows<L>::bytes_per_walker() + PairRing<L, TRIES>::bytes());
     static std::atomic<uint64_t> allowed{0};
-    const cudaError_t err = allow_smem(pair_kernel<L>, allowed);
+    const cudaError_t err = allow_smem(pair_kernel<L, TRIES>, allowed);
     if (err != cudaSuccess)
         return err;
     LaunchPlan plan;
@@ -299,7 +300,7 @@ cudaError_t launch_pair_t(const SweepArgs &a, int chains, bool record, cudaStrea
     plan.phase[1] = row_plan(L, a.t0 + a.n_therm, a.n);
     const int gens = chains == 1 ? 2 : 1;
     const int64_t blocks = (a.W + 32 * chains - 1) / (32 * chains);
-    pair_kernel<L><<<(unsigned)blocks, 32 * chains * (1 + gens), smem, s>>>(a, plan, chains, gens, record);
+    pair_kernel<L, TRIES><<<(unsigned)blocks, 32 * chains * (1 + gens), smem, s>>>(a, plan, chains, gens, record);
     return cudaGetLastError();
 }
 
