@@ -48,10 +48,10 @@ MAX_ITERATIONS = 2 * 10**4 * L_SIDE * L_SIDE // (WALKERS * SWEEPS_PER_ITER)   # 
 # load, compare, conditional flip, energy update, run-length histogram record, about
 # 15.5).  Fixed by the method, not measured from the code.
 OPS_PER_ATTEMPT = 35.0
-# Warp instructions the step's whole-sweep launch issues per attempt and warp (ncu
+# Warp instructions the step's sweep launch issues per attempt and warp (ncu
 # count, profiles/sweep_full_kernel_L32_W16384_int8.md): converts an instruction issue
 # rate into this roofline's algorithmic operations.
-INSTR_PER_ATTEMPT = 31.13
+INSTR_PER_ATTEMPT = 28.82
 WORKLOAD = (f"muca2d_ising_L{L_SIDE}_W{WALKERS}_int8_therm{THERM_SWEEPS}_rec{SWEEPS_PER_ITER}")
 
 
@@ -197,7 +197,7 @@ class ClockSampler:
         return {"sm_mhz": sm[len(sm) // 2], "sm_max_mhz": mx, "reasons": sorted(reasons), "samples": len(sm)}
 
 
-# Sources that define the timed whole-sweep kernel at L = 32 (body and launcher).
+# Sources that define the timed sweep kernel at L = 32 (body and launcher).
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_1707_00919_gb300", "csrc", f)
                   for f in ("muca_device.cuh", "muca_full.cuh", "muca_full_32.cu")]
 TRAFFIC_PROFILE = os.path.join(ROOT, "profiles", "sweep_full_kernel_L32_W16384_int8.md")
@@ -530,7 +530,7 @@ def run_native(args):
         "gpu_launches": 2 * args.steps,   # per step: table_kernel, sweep_full_kernel
         "roofline": {"bound": "alu", "achieved": achieved_tops, "peak": peak_tops, "unit": "Tops/s (int32)",
                      "frac": achieved_tops / peak_tops, "traffic": traffic,
-                     "kernel": "sweep_full_kernel<32,int8,record> (31 thermalization + 10 recorded "
+                     "kernel": "sweep_full_kernel<32, AttemptStream<32, 7, 1>> (31 thermalization + 10 recorded "
                                "sweeps in one launch)",
                      "ops_per_attempt": OPS_PER_ATTEMPT,
                      "peak_basis": f"{sm_count} SMs x 4 issue slots x 32 lanes x {sm_max_mhz:.0f} MHz",

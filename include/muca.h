@@ -297,9 +297,10 @@ int muca_reset_histogram(muca_t h);
  * N_updates recorded ones): zeroes H, then every walker performs n_therm attempts
  * without recording and n_record recorded attempts.  The results (lattices, energies,
  * attempt counter, H) equal those of muca_reset_histogram, muca_attempts(h, n_therm, 0)
- * and muca_attempts(h, n_record, 1).  In typewriter order, when both counts are whole
- * sweeps starting at a sweep boundary, the two phases run in one kernel launch (the
- * lattices are read and written once); otherwise as two launches.  Asynchronous. */
+ * and muca_attempts(h, n_record, 1).  In typewriter order, when neither count is zero, the two
+ * phases run in one kernel launch (the lattices are read and written once) unless n_record
+ * exceeds what a launch can count (0xFFFFFFFF / 256 attempts per walker) or the range crosses
+ * a multiple of 2^34 attempts; otherwise as two launches or more.  Asynchronous. */
 int muca_thermalize_and_record(muca_t h, uint64_t n_therm, uint64_t n_record);
 
 /* The weight iteration of Sec. 2.2 and Sec. 3: repeat { thermalize; zero H; record;
@@ -393,8 +394,8 @@ int muca_philox(const uint32_t *ctr, const uint32_t key[2], size_t n, uint32_t *
 /* ----------------------------------------------------------------------------------
  * Batches (Sec. 2.2 applied to many independent simulations at once): one launch of a
  * persistent kernel advances every member instance; each block takes work items
- * (instance, 256 or fewer walkers) from a global counter, so instances of uneven L and
- * walker count share the GPU.  Member instances must have L in {8, 16, 24, 32, 48, 64}.
+ * (instance, 256 or fewer walkers) from one list, so instances of uneven L and walker count
+ * share the GPU.  Member instances must have L in {8, 16, 24, 32, 48, 64}.
  * Results are the same as running each instance alone (walkers and histograms of
  * different instances never interact).
  * -------------------------------------------------------------------------------- */

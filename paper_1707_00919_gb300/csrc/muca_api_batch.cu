@@ -43,8 +43,9 @@ namespace {
 bool batchable_L(int32_t L) { return L == 8 || L == 16 || L == 24 || L == 32 || L == 48 || L == 64; }
 
 // Time of an item of `walkers` walkers and `length` attempts each, in cycles: a block has an
-// SM to itself, so an attempt's time goes by the warps that share a sub-partition (L = 64:
-// 59 cycles alone, 93 for two), whether all their lanes hold walkers or not.
+// SM to itself, so an attempt's time goes by the warps that share a sub-partition (measured at
+// L = 64, the size of the longest items, and taken for all: 59 cycles alone, 93 for two),
+// whether all their lanes hold walkers or not.
 double item_time(uint64_t length, int64_t walkers)
 {
     const int64_t warps = (walkers + 31) / 32, share = (warps + 3) / 4;

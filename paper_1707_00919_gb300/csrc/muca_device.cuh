@@ -1,6 +1,6 @@
-// muca_device.cuh - device code of the whole-sweep kernels, shared by the per-L
-// translation units (muca_full_L.cu), the batched kernels (muca_batch.cu) and the
-// generic kernels (muca_kernels.cu).  Parallel multicanonical 2D Ising update of Gross,
+// muca_device.cuh - device code of the sweep kernels, shared by the per-L translation units
+// (muca_full_L.cu), the batched kernels (muca_batch.cu, muca_noalloc.cu), the kernel of the
+// random site order (muca_random.cu) and those around the sweeps (muca_kernels.cu).  Parallel multicanonical 2D Ising update of Gross,
 // Zierenberg, Weigel, Janke (arXiv:1707.00919), Sec. 2.3.
 #pragma once
 
@@ -448,7 +448,7 @@ __device__ __forceinline__ uint32_t add_count(uint32_t w, int x, int m, uint32_t
 }
 
 // ---------------------------------------------------------------------------------
-// Continuous attempt stream over whole rows (whole-sweep launches).  The two threshold
+// Continuous attempt stream over the whole rows of a range.  The two threshold
 // candidates of every attempt are loaded two attempts ahead, across row ends as well:
 // the first two sites of the next row have as neighbours the current row's first two
 // sites (final after its attempts 0 and 1) and rows that the current row does not
@@ -471,8 +471,10 @@ __device__ __forceinline__ uint32_t add_count(uint32_t w, int x, int m, uint32_t
 //   L = 32, 4096 walkers, chain warps with generators       18.7 / 18.2 / 17.7
 //   L = 64, 4096 walkers, the same                          74.8 / 74.2 / 72.1
 //   L = 8, 128 walkers, the same                            1.23 / 1.16 / 1.28
-// (24.9 at 16 384 walkers with selects and exclusive-ors for the flips and the reduction
-// first; 25.6 with shifted and masked count fields, 31.1 instructions per attempt.)
+// (side by side, before the lattices' and the table's loads took their present form: the
+// chain warps of L = 64 now take 73.4.  At 16 384 walkers 24.9 with selects and exclusive-ors
+// for the flips and the reduction first; 25.6 with shifted and masked count fields, 31.1
+// instructions per attempt.)
 // ---------------------------------------------------------------------------------
 template <int L, int STRIDE, int EARLY>
 struct AttemptStream {
@@ -566,8 +568,8 @@ struct AttemptStream {
 // ---------------------------------------------------------------------------------
 // The same rows without the look-ahead: each attempt loads its one threshold once the
 // attempt before it is decided.  The chain of an attempt (address, load, compare, select)
-// then holds the load's latency, which other warps have to cover, but an attempt is 22.5
-// instructions instead of 27.2.  The decision enters as a factor 0 or 1: the step of the
+// then holds the load's latency, which other warps have to cover, but an attempt is 22.8
+// instructions instead of 28.6 (L = 32, counted by ncu over 20 sweeps).  The decision enters as a factor 0 or 1: the step of the
 // energy row and the flip bit are multiply-adds, on the pipe with room, where a select
 // each would load the ALU.  Measured at L = 32, 48 640 walkers (2.5 warps per SM
 // sub-partition) 57.9 us per sweep against 61.5 with the look-ahead; L = 16, 77 824 walkers

@@ -60,11 +60,11 @@ constexpr size_t kEnergyStageBytes = 256 * 1024;
 // shared histogram bins cannot overflow (each walker adds one count per attempt).
 inline uint64_t max_recorded_attempts(int wpb) { return 0xFFFFFFFFull / (uint64_t)std::max(wpb, 256); }
 
-// Sweeps of an instance, a batch or allocation-free calls, queued on a device and perhaps still running, so that a launch knows whether it has
-// the device to itself (launch_sweep's form; results do not depend on it).  What says that
-// they have ended is their stream, where it is the library's own and outlives the flight,
-// else an event behind them: a caller's stream may be gone or under capture when another
-// instance asks, and may run the caller's own work.
+// Sweeps of an instance, a batch or allocation-free calls, queued on a device and perhaps still
+// running, so that a launch knows whether it has the device to itself (launch_sweep's form;
+// results do not depend on it).  What says that they have ended is their stream, where it is
+// the library's own and outlives the flight, else an event behind them: a caller's stream may
+// be gone or under capture when another instance asks, and may run the caller's own work.
 struct Flight {
     int device = 0;
     int company = 0;               // launches for which it is taken to overlap others
@@ -143,7 +143,7 @@ int sync_and_check(muca_t h);
 cudaError_t wait_stream(muca_t h);
 int run_attempts(muca_t h, uint64_t n, bool record, const uint32_t *skip = nullptr);
 // n_therm attempts without recording, then n_record recorded ones (the histogram is not
-// zeroed here); one kernel launch where the whole-sweep kernel allows it.
+// zeroed here); one kernel launch in typewriter order (run_therm_record).
 int run_therm_record(muca_t h, uint64_t n_therm, uint64_t n_record, const uint32_t *skip = nullptr);
 int read_histogram(muca_t h, std::vector<uint64_t> &H);
 // The instance's histogram, or its sum over the instances of the simulation when a reducer is set.

@@ -10,7 +10,7 @@
 
 namespace muca {
 
-// Shared-memory table of the whole-sweep kernels: one row of kTableStride words per
+// Shared-memory table of the sweep kernels: one row of kTableStride words per
 // energy, thresholds in words 0..4, the block's histogram count in word kHistSlot.
 constexpr int kTableStride = 7;
 constexpr int kHistSlot = 5;

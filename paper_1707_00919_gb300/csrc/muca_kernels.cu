@@ -182,8 +182,8 @@ __global__ void philox_kernel(const uint32_t *ctr, uint32_t k0, uint32_t k1, siz
 // The form of a launch by the warps of walkers per SM.  Up to two, and with the device to
 // itself: the paired kernel, its generator warps on the sub-partitions that would idle
 // (when sweeps of other instances run, it would take SMs from them for less throughput:
-// eight instances of L = 32 with 4096 walkers, all queued, 1661 us per 20 sweeps with it
-// against 955).  Up to eight, two per sub-partition: the two-ahead loads.  More than that
+// eight instances of L = 32 with 4096 walkers, all queued, 1724 us per 20 sweeps with it
+// against 890).  Up to eight, two per sub-partition: the two-ahead loads.  More than that
 // resident at once: direct loads, whose latency the other warps cover (how many the kernel's
 // blocks leave resident is looked at where it is launched, muca_full.cuh).
 SweepForm sweep_form(const SweepArgs &a, bool alone)

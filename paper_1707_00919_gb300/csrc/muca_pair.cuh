@@ -7,9 +7,9 @@
 // draw the words into a ring in shared memory, a chunk of about 128 attempts at a time, and
 // the chain warp reads four words per 16-byte load.  What bounds it now is the chain warp's
 // issue again, 18 instructions per attempt.  Measured, us per sweep without and with the
-// generators: L = 8, 128 walkers 1.58 -> 1.19; L = 16, 4096 walkers 6.31 -> 4.41; L = 24,
-// 5003 walkers 14.2 -> 10.4; L = 32, 4096 walkers 24.5 -> 17.7; L = 48, 1024 walkers 56.6 ->
-// 42.2; L = 64, 9728 walkers 99.6 -> 73.4.
+// generators: L = 8, 128 walkers 1.58 -> 1.19; L = 16, 4096 walkers 6.30 -> 4.41; L = 24,
+// 5003 walkers 14.2 -> 10.4; L = 32, 4096 walkers 24.4 -> 17.7; L = 48, 1024 walkers 56.5 ->
+// 42.0; L = 64, 4096 or 9728 walkers 99.4 -> 73.4.
 #pragma once
 
 #include "muca_device.cuh"
@@ -50,7 +50,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
 // (c), so that both sides agree on slot and phase.
 template <int L, uint32_t TRIES>
 struct PairRing {
-    static constexpr int kRows = L < 128 ? 128 / L : 1;             // rows per chunk
+    static constexpr int kRows = 128 / L;                           // rows per chunk
     static constexpr int kTogether = 4;                             // blocks drawn together
     static constexpr int kBlocks = (kRows * (L / 4) + kTogether - 1) / kTogether * kTogether;
     static constexpr uint32_t kSlotBytes = kBlocks * 512;
